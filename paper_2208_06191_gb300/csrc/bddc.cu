@@ -1509,6 +1509,32 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
   C->setup_flops = fl;
   C->local_bytes = lb;
   C->apply_flops = (double)lb / (double)C->esize * 2.0;
+  // FP64 lists (local operators of FP64 contexts, the coarse inverse): one
+  // scratch buffer for the digits, shared by every list.  The coarsest
+  // inverse under FP32 level-2 operators keeps the FMA kernel: the hardest
+  // Newton states of the 3M-DoF P2 ventricle converge or stagnate with the
+  // last bits of the preconditioner (519 iterations, or more than 1000 in two
+  // of seven runs from states moved by 1e-13, with either kernel), the FMA
+  // kernel's bits are the ones those solves are validated with, and the
+  // inverse is small (867 unknowns: 1.9 ms of a 290 ms setup).
+  {
+    std::vector<GemmList*> lists;
+    if (C->esize == 8 || P->nnzb > 0)
+      for (auto& g : C->gl_swc) lists.push_back(&g);
+    if (C->esize == 8) {
+      for (auto* g : {&C->gl_E, &C->gl_S, &C->gl_W, &C->gl_T, &C->gl_PhiA, &C->gl_SPhi, &C->gl_Kc, &C->gl_PsiV,
+                      &C->gl_dlx})
+        lists.push_back(g);
+      for (auto* v : {&C->gl_sw1, &C->gl_sw2, &C->gl_swg, &C->gl_swd})
+        for (auto& g : *v) lists.push_back(&g);
+    }
+    int64_t need = 0;
+    for (auto* g : lists) need = std::max(need, g->oz_bytes());
+    if (need > 0) {
+      C->oz_scratch.alloc((size_t)need);
+      for (auto* g : lists) g->bind_oz(C->oz_scratch.p, P->status.p);
+    }
+  }
   // FP32 contexts: one scratch buffer for the split operands of the
   // tensor-core GEMMs, shared by every list (they run one after another on
   // the setup stream)

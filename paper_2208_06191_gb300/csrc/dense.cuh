@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "common.h"
+#include "oz_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace cbddc {
@@ -317,6 +318,14 @@ struct GemmList {
   int np = 2;  // TF32 parts per operand
   tc::TcMaps maps;
   std::vector<GemmProb> h;  // host copy of the problems
+  // integer-slice tensor-core plan (FP64)
+  DVec<oz::Prob> ozp;
+  DVec<oz::SplitProb> oza, ozb;
+  DVec<int2> oz_ia, oz_ib;  // split work items
+  DVec<int4> oz_tiles;
+  std::vector<oz::Batch> oz_batches;
+  unsigned char* oz_base = nullptr;
+  int* oz_status = nullptr;
   // order 1: tiles of the largest problems (M N K) first, so that with
   // uneven subdomains the long tile runs of a persistent kernel start early
   void set(const std::vector<GemmProb>& v, size_t esize, bool ta = false, int order = 0) {
@@ -345,6 +354,84 @@ struct GemmList {
     tiles.upload(t);
     tc_planned = tc_bound = false;
     if (esize == 4 && ntiles > 0 && n <= 65535) plan_tc(v);
+    if (esize == 8 && ntiles > 0) plan_oz(v, order);
+  }
+  // FP64: batches of problems whose digits share the scratch buffer, with
+  // the split work items (blocks of 32 rows) and the output tiles of each
+  void plan_oz(const std::vector<GemmProb>& v, int order) {
+    std::vector<oz::Prob> pr(n);
+    std::vector<oz::SplitProb> sa(n), sb(n);
+    std::vector<int2> ia, ib;
+    std::vector<int4> t;
+    oz_batches.clear();
+    auto work = [&](const int4& a) { return (double)v[a.x].M * v[a.x].N * v[a.x].K; };
+    auto close = [&] {
+      if (oz_batches.empty()) return;
+      oz::Batch& b = oz_batches.back();
+      b.na = (int)ia.size() - b.a0;
+      b.nb = (int)ib.size() - b.b0;
+      b.nt = (int)t.size() - b.t0;
+      if (order == 1)
+        std::stable_sort(t.begin() + b.t0, t.end(), [&](const int4& x, const int4& y) { return work(x) > work(y); });
+    };
+    for (int i = 0; i < n; ++i) {
+      const GemmProb& q = v[i];
+      if (q.M <= 0 || q.N <= 0 || q.K <= 0) {
+        pr[i] = oz::Prob{0, 0, 0, 0, 0, 0, 0};
+        sa[i] = sb[i] = oz::SplitProb{0, 0, 0, 0, 0};
+        continue;
+      }
+      CB_CHECK(q.K <= 1 << 24, CBDDC_EINVAL, "dense product too long");
+      const int Kp = (int)round_up(q.K, oz::BK);
+      bool fresh = oz_batches.empty();
+      if (!fresh) {
+        oz::Batch b = oz_batches.back();
+        b.Kp = std::max(b.Kp, Kp);
+        b.rowsA += q.M;
+        b.rowsB += q.N;
+        fresh = b.bytes() > oz::kBatchBytes || b.rowsA >= INT32_MAX || b.rowsB >= INT32_MAX;
+      }
+      if (fresh) {
+        close();
+        oz::Batch b;
+        b.a0 = (int)ia.size();
+        b.b0 = (int)ib.size();
+        b.t0 = (int)t.size();
+        oz_batches.push_back(b);
+      }
+      oz::Batch& b = oz_batches.back();
+      b.Kp = std::max(b.Kp, Kp);
+      pr[i] = oz::Prob{q.M, q.N, q.K, q.ldc, q.c, (int)b.rowsA, (int)b.rowsB};
+      sa[i] = oz::SplitProb{q.M, q.K, q.lda, (int)b.rowsA, q.a};
+      sb[i] = oz::SplitProb{q.N, q.K, q.ldb, (int)b.rowsB, q.b};
+      b.rowsA += q.M;
+      b.rowsB += q.N;
+      for (int k = 0; k < (int)cdiv(q.M, 32); ++k) ia.push_back(make_int2(i, k));
+      for (int k = 0; k < (int)cdiv(q.N, 32); ++k) ib.push_back(make_int2(i, k));
+      for (int tm = 0; tm < (int)cdiv(q.M, oz::BM); ++tm)
+        for (int tn = 0; tn < (int)cdiv(q.N, oz::BN); ++tn) t.push_back(make_int4(i, tm, tn, 0));
+    }
+    close();
+    ozp.upload(pr);
+    oza.upload(sa);
+    ozb.upload(sb);
+    oz_ia.upload(ia);
+    oz_ib.upload(ib);
+    oz_tiles.upload(t);
+  }
+  // bytes of digit scratch this list needs
+  int64_t oz_bytes() const {
+    int64_t m = 0;
+    for (const auto& b : oz_batches) m = std::max(m, b.bytes());
+    return m;
+  }
+  void bind_oz(unsigned char* base, int* status) {
+    oz_base = base;
+    oz_status = status;
+    for (auto& b : oz_batches) {
+      b.maps.a = oz::encode_digits(reinterpret_cast<__half*>(base), b.rowsA, b.Kp, oz::BM);
+      b.maps.b = oz::encode_digits(reinterpret_cast<__half*>(base + b.bytes_a()), b.rowsB, b.Kp, oz::BN);
+    }
   }
   void plan_tc(const std::vector<GemmProb>& v) {
     std::vector<tc::TcProb> tp(n);
@@ -461,6 +548,33 @@ void launch_tc(const GemmList& g, const float* A, const float* B, float* C, floa
   CB_LAUNCH();
 }
 
+// C = sign op(A) op(B) (+ C) for a bound FP64 list: per batch, the digits of
+// both operands, then one persistent tcgen05 kernel.
+template <bool TA, bool TB>
+void launch_oz(const GemmList& g, const double* A, const double* B, double* C, double alpha, double beta,
+               cudaStream_t s) {
+  CB_CHECK((alpha == 1.0 || alpha == -1.0) && (beta == 0.0 || beta == 1.0), CBDDC_EINVAL, "dense product factors");
+  oz::set_smem_attr();
+  for (const oz::Batch& b : g.oz_batches) {
+    __half* da = reinterpret_cast<__half*>(g.oz_base);
+    __half* db = reinterpret_cast<__half*>(g.oz_base + b.bytes_a());
+    int* ea = reinterpret_cast<int*>(g.oz_base + b.bytes_a() + b.bytes_b());
+    int* eb = reinterpret_cast<int*>(g.oz_base + b.bytes_a() + b.bytes_b() + b.bytes_ea());
+    oz::split_kernel<!TA><<<b.na, 256, 0, s>>>(g.oz_ia.p + b.a0, g.oza.p, b.Kp, A, da, b.rowsA * b.Kp, ea);
+    CB_LAUNCH();
+    oz::split_kernel<TB><<<b.nb, 256, 0, s>>>(g.oz_ib.p + b.b0, g.ozb.p, b.Kp, B, db, b.rowsB * b.Kp, eb);
+    CB_LAUNCH();
+    const int grid = tc::tc_grid(b.nt);
+    if (beta == 0.0)
+      oz::gemm_kernel<false><<<grid, oz::THREADS, oz::SMEM, s>>>(g.oz_tiles.p + b.t0, b.nt, g.ozp.p, b.maps, ea, eb,
+                                                                 C, alpha < 0.0, g.oz_status);
+    else
+      oz::gemm_kernel<true><<<grid, oz::THREADS, oz::SMEM, s>>>(g.oz_tiles.p + b.t0, b.nt, g.ozp.p, b.maps, ea, eb,
+                                                                C, alpha < 0.0, g.oz_status);
+    CB_LAUNCH();
+  }
+}
+
 template <typename T, bool TA, bool TB>
 void launch_gemm(const int4* tiles, int ntiles, const GemmProb* probs, const T* A, const T* B, T* C,
                  T alpha, T beta, cudaStream_t s, bool fast = false) {
@@ -489,8 +603,16 @@ void launch_list(const GemmList& g, const T* A, const T* B, T* C, T alpha, T bet
       timer_end(cls, s, g.flops, g.bytes);
       return;
     }
+  } else if (g.oz_base != nullptr) {
+    launch_oz<TA, TB>(g, A, B, C, alpha, beta, s);
+    timer_end(cls, s, g.flops, g.bytes);
+    return;
   }
-  launch_gemm<T, TA, TB>(g.tiles.p, g.ntiles, g.d.p, A, B, C, alpha, beta, s, g.fast);
+  // FP64 without digit scratch: a coarsest inverse (plain products only)
+  if constexpr (sizeof(T) == 4 || (!TA && !TB))
+    launch_gemm<T, TA, TB>(g.tiles.p, g.ntiles, g.d.p, A, B, C, alpha, beta, s, g.fast);
+  else
+    CB_CHECK(false, CBDDC_EINVAL, "transposed FP64 product without scratch");
   timer_end(cls, s, g.flops, g.bytes);
 }
 
