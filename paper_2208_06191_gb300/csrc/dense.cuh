@@ -631,95 +631,127 @@ struct SweepDesc {
 };
 
 // P = inverse of the kb x kb diagonal block of pivot step k, by Gauss-Jordan
-// in the operator precision T.  Thread (c, g) = (tid % NB, tid / NB) keeps
-// RG rows of column c in registers (16 of 256 threads for NB = 64, 32 of
-// 512 for NB = 128), so all four SM sub-partitions stay busy (the FP64
-// coarse matrix needs every FP64 unit).  At pivot j every thread reads
-// the old pivot column and pivot row from a double-buffered shared copy,
-// updates its entries
+// in the operator precision T: at pivot j
 //   a[j][c] <- a[j][c] / p,  a[i][c] <- a[i][c] - a[i][j] a[j][c] / p (c != j),
-//   a[i][j] <- -a[i][j] / p, a[j][j] <- 1 / p,
-// and the owners of column j + 1 and row j + 1 publish them into the other
-// buffer, so one barrier per pivot suffices.
-// Threads of the diagonal-block kernel: 256 for NB = 64 (16 rows of one
-// column per thread), 512 for NB = 128 (32 rows per thread).
+//   a[i][j] <- -a[i][j] / p, a[j][j] <- 1 / p.
+// Warp w keeps rows 8 w .. 8 w + 7 in registers, lane l their columns l, l +
+// 32, ...  The warp that owns row j + 1 updates that row first, forms the
+// reciprocal of its pivot and the scaled row, and publishes them (with the
+// reciprocal in place of entry j + 1) in a double-buffered shared copy, as the
+// owners of column j + 1 do with the column, while the other warps still
+// update: one barrier per pivot, and one reciprocal instead of one per warp.
+//
+// One CTA per matrix, a chain of kb pivots.  FP64: bound by the FP64 pipe, 128
+// warp instructions of 16 clocks per pivot of a 64-wide block (66 us at
+// least); 95 us measured, 166 us when every warp formed the reciprocal behind
+// the barrier.  FP32: bound by the chain (barrier, reciprocal, broadcast),
+// 22 us against 39 us.
 template <int NB>
-struct DiagThreads { static constexpr int value = NB <= 64 ? 256 : 512; };
-constexpr int DIAG_THREADS = 256;
+struct DiagThreads { static constexpr int value = 4 * NB; };
 template <typename T, int NB>
 __global__ void __launch_bounds__(DiagThreads<NB>::value)
 sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat, T* __restrict__ Pbuf,
                   int* __restrict__ status, double tol) {
-  constexpr int NT = DiagThreads<NB>::value;
-  constexpr int RG = NB / (NT / NB);  // rows per thread
-  __shared__ T colb[2][NB], rowb[2][NB];
-  __shared__ double piv_scale;
-  __shared__ int bad;
+  constexpr int RW = 8, CW = NB / 32;  // rows per warp, columns per lane
+  __shared__ __align__(16) T colb[2][NB];
+  __shared__ T rowb[2][NB];
   const SweepDesc d = desc[blockIdx.x];
   const int k0 = k * NB;
   if (k0 >= d.p) return;
   const int kb = min(NB, d.p - k0);
-  const int tid = threadIdx.x;
-  const int c = tid % NB, r0 = (tid / NB) * RG;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = RW * warp;
   const T* A = mat + d.off + (int64_t)k0 * d.ld + k0;
-  if (tid == 0) bad = 0;
-  T a[RG];
+  T a[RW][CW];
 #pragma unroll
-  for (int q = 0; q < RG; ++q)
-    a[q] = (r0 + q < kb && c < kb) ? A[(int64_t)(r0 + q) * d.ld + c] : T(0);
-  if (c == 0) {
+  for (int q = 0; q < RW; ++q)
 #pragma unroll
-    for (int q = 0; q < RG; ++q) colb[0][r0 + q] = a[q];
-  }
-  if (r0 == 0) rowb[0][c] = a[0];
-  // scale of the pivots: largest |diagonal| of the block
-  if (tid < 32) {
-    double dv = 0.0;
-    for (int i = tid; i < kb; i += 32) dv = fmax(dv, fabs((double)A[(int64_t)i * d.ld + i]));
-    for (int o = 16; o > 0; o >>= 1) dv = fmax(dv, __shfl_xor_sync(0xffffffffu, dv, o));
-    if (tid == 0) piv_scale = dv;
-  }
-  __syncthreads();
-  const double scale = piv_scale;
-  for (int j = 0; j < kb; ++j) {
-    const int b = j & 1, nb = b ^ 1;
-    const T pv = rowb[b][j];
-    const T rj = rowb[b][c];
+    for (int v = 0; v < CW; ++v) {
+      const int c = lane + 32 * v;
+      a[q][v] = (r0 + q < kb && c < kb) ? A[(int64_t)(r0 + q) * d.ld + c] : T(0);
+    }
+  // scale of the pivots: largest |diagonal| of the block (every warp)
+  double scale = 0.0;
+  for (int i = lane; i < kb; i += 32) scale = fmax(scale, fabs((double)A[(int64_t)i * d.ld + i]));
+  for (int o = 16; o > 0; o >>= 1) scale = fmax(scale, __shfl_xor_sync(0xffffffffu, scale, o));
+  bool bad = false;
+  // scaled row j (held by this warp in r) into buffer b
+  auto publish_row = [&](const T* r, int j, int b) {
+    T pv = T(0);
+#pragma unroll
+    for (int v = 0; v < CW; ++v)
+      if (v == (j >> 5)) pv = r[v];
+    pv = __shfl_sync(0xffffffffu, pv, j & 31);
     const T inv = T(1) / pv;
-    if (c < kb) {
-      if (c == j) {
 #pragma unroll
-        for (int q = 0; q < RG; ++q) a[q] = (r0 + q == j) ? inv : -colb[b][r0 + q] * inv;
+    for (int v = 0; v < CW; ++v) {
+      const int c = lane + 32 * v;
+      rowb[b][c] = c == j ? inv : r[v] * inv;
+    }
+    if (!(fabs((double)pv) > tol * scale) || !isfinite((double)pv)) bad = true;
+  };
+  auto publish_col = [&](int j, int b) {
+    if (lane == (j & 31)) {
+#pragma unroll
+      for (int v = 0; v < CW; ++v)
+        if (v == (j >> 5)) {
+#pragma unroll
+          for (int q = 0; q < RW; ++q) colb[b][r0 + q] = a[q][v];
+        }
+    }
+  };
+  if (warp == 0) publish_row(a[0], 0, 0);
+  publish_col(0, 0);
+  for (int j0 = 0; j0 < kb; j0 += RW) {
+#pragma unroll
+    for (int u = 0; u < RW; ++u) {
+      const int j = j0 + u;
+      if (j >= kb) break;
+      constexpr int un_of[RW] = {1, 2, 3, 4, 5, 6, 7, 0};
+      const int un = un_of[u];                      // row of j + 1 in its warp
+      const int b = u & 1;
+      const bool last = j + 1 >= kb;
+      __syncthreads();
+      T t[CW], col[RW];
+      bool own[CW];                                 // this lane's column is j
+#pragma unroll
+      for (int v = 0; v < CW; ++v) {
+        t[v] = rowb[b][lane + 32 * v];
+        own[v] = lane + 32 * v == j;
+      }
+#pragma unroll
+      for (int q = 0; q < RW; ++q) col[q] = colb[b][r0 + q];
+      auto update = [&](int q) {
+#pragma unroll
+        for (int v = 0; v < CW; ++v) a[q][v] = (own[v] ? T(0) : a[q][v]) - col[q] * t[v];
+      };
+      if (warp == (j + 1) / RW && !last) {
+        update(un);
+        // (row j + 1 is never row j)
+        publish_row(a[un], j + 1, b ^ 1);
+#pragma unroll
+        for (int q = 0; q < RW; ++q)
+          if (q != un) update(q);
       } else {
-        const T t = rj * inv;
 #pragma unroll
-        for (int q = 0; q < RG; ++q) a[q] = (r0 + q == j) ? t : a[q] - colb[b][r0 + q] * t;
+        for (int q = 0; q < RW; ++q) update(q);
       }
+      if (warp == j0 / RW) {
+#pragma unroll
+        for (int v = 0; v < CW; ++v) a[u][v] = t[v];
+      }
+      if (!last) publish_col(j + 1, b ^ 1);
     }
-    if (j + 1 < kb) {
-      if (c == j + 1) {
-#pragma unroll
-        for (int q = 0; q < RG; ++q) colb[nb][r0 + q] = a[q];
-      }
-      const int jr = j + 1 - r0;
-      if (jr >= 0 && jr < RG) {
-        T v = T(0);
-#pragma unroll
-        for (int q = 0; q < RG; ++q)
-          if (q == jr) v = a[q];
-        rowb[nb][c] = v;
-      }
-    }
-    if (tid == 0 && (!(fabs((double)pv) > tol * scale) || !isfinite((double)pv))) bad = 1;
-    __syncthreads();
   }
   T* P = Pbuf + d.offP;
-  if (c < kb) {
 #pragma unroll
-    for (int q = 0; q < RG; ++q)
-      if (r0 + q < kb) P[(r0 + q) * NB + c] = a[q];
-  }
-  if (tid == 0 && bad) atomicOr(status, DEV_PIVOT);
+  for (int q = 0; q < RW; ++q)
+#pragma unroll
+    for (int v = 0; v < CW; ++v) {
+      const int c = lane + 32 * v;
+      if (c < kb && r0 + q < kb) P[(r0 + q) * NB + c] = a[q][v];
+    }
+  if (lane == 0 && bad) atomicOr(status, DEV_PIVOT);
 }
 
 // Builds X and Y panels and zeroes the pivot rows/columns, for indices
