@@ -51,13 +51,6 @@ constexpr int SMEM = S * (A_BYTES + B_BYTES) + 1024 /* alignment */ + 512 /* bar
 static_assert(SMEM <= 232448, "shared memory per CTA");
 constexpr int EXP_NAN = 0x7fffff;  // row exponent of a row with a non-finite entry
 
-// One lane of a converged warp.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t e;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
-  return e != 0;
-}
-
 // kind::f16 instruction descriptor: D = F32 (bits 4-5), A = B = F16 (0),
 // both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
 constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -345,7 +338,7 @@ gemm_kernel(const int4* __restrict__ tiles, int ntiles, const Prob* __restrict__
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t acc = tmem + (uint32_t)(a * BN);
-          if (elect_one()) {
+          if (tc::elect_one()) {
             // descriptors differ in their address field only (16-byte units)
 #pragma unroll
             for (int x = 0; x <= k; ++x) {

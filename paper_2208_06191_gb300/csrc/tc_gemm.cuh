@@ -128,6 +128,13 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
       : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+
 // Arrives on bar once every tcgen05.mma issued so far by this thread is done.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -209,7 +216,7 @@ struct TcMaps {
 //
 // Warp roles (320 threads):
 //   warp 0, one lane: TMA producer of the operand chunks (NST-stage ring);
-//   warp 1, one lane: MMA issuer; chunk g of the CTA goes to TMEM slice g % 2;
+//   warp 1: MMA issuer (one elected lane); chunk g of the CTA goes to TMEM slice g % 2;
 //   warps 2-9: epilogue; warp w reads TMEM lanes (tile rows) 32 (w % 4) ..
 //     + 31 and column half (w - 2) / 4 (64 columns), adds every chunk's
 //     slice into 64 FP32 running sums per thread and frees the slice; at the
@@ -237,7 +244,8 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
   uint64_t* sempty = sfull + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sempty + 2);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (the shuffle tells the compiler that the warp number is uniform)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int ntl = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (threadIdx.x == 0) {
@@ -291,34 +299,39 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int g = 0;  // TMEM slices of this CTA so far (SPC per operand chunk)
-      bool ok = true;
-      for (int i = 0; i < ntl && ok && !*(volatile int*)abort_flag; ++i) {
-        const int4 tl = tiles[blockIdx.x + i * gridDim.x];
-        const int nk = (probs[tl.x].K + BKC - 1) / BKC;
-        for (int c = 0; c < nk; ++c) {
-          const int s = (g / SPC) % NST;  // operand stage of chunk c (g counts slices)
-          if (!mbar_wait(&full[s], ((g / SPC) / NST) & 1)) {
+    // The whole warp walks the loop and one lane issues, so that the operands
+    // of the MMAs stay in uniform registers (with the loop under a single
+    // lane every MMA cost about 100 clocks).
+    int g = 0;  // TMEM slices of this CTA so far (SPC per operand chunk)
+    bool ok = true;
+    for (int i = 0; i < ntl && ok && !*(volatile int*)abort_flag; ++i) {
+      const int4 tl = tiles[blockIdx.x + i * gridDim.x];
+      const int nk = (probs[tl.x].K + BKC - 1) / BKC;
+      for (int c = 0; c < nk && ok; ++c) {
+        const int s = (g / SPC) % NST;  // operand stage of chunk c (g counts slices)
+        if (!mbar_wait(&full[s], ((g / SPC) / NST) & 1)) {
+          ok = false;
+          break;
+        }
+        // parts: a_q at tile q, b_q at tile NP + q (addresses in 16-byte units)
+        const uint64_t d0 = sw128_desc(smem_u32(smem + s * STAGE_BYTES));
+#pragma unroll
+        for (int sl = 0; sl < SPC; ++sl, ++g) {
+          const int a = g & 1;
+          if (!ok) break;
+          if (g >= 2 && !mbar_wait(&sempty[a], ((g >> 1) - 1) & 1)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t st = smem_u32(smem + s * STAGE_BYTES);
-          for (int sl = 0; sl < SPC && ok; ++sl, ++g) {
-            const int a = g & 1;
-            if (g >= 2 && !mbar_wait(&sempty[a], ((g >> 1) - 1) & 1)) {
-              ok = false;
-              break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t acc = tmem + (uint32_t)(a * TMEM_COLS);
+          const uint32_t acc = tmem + (uint32_t)(a * TMEM_COLS);
+          if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk) {
               const int k = sl * KS + kk;
-              // parts: a_q at tile q, b_q at tile NP + q; small products first
-              auto da = [&](int q) { return sw128_desc(st + q * OPND_BYTES + 32 * k); };
-              auto db = [&](int q) { return sw128_desc(st + (NP + q) * OPND_BYTES + 32 * k); };
+              // small products first
+              auto da = [&](int q) { return d0 + (uint32_t)(q * (OPND_BYTES / 16) + 2 * k); };
+              auto db = [&](int q) { return d0 + (uint32_t)((NP + q) * (OPND_BYTES / 16) + 2 * k); };
               const uint32_t first = kk > 0 ? 1u : 0u;  // each slice starts afresh
               if (NP == 3) {
                 mma_tf32(acc, da(1), db(1), first);
@@ -332,14 +345,13 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
               mma_tf32(acc, da(0), db(0), 1u);
             }
             mma_commit(&sfull[a]);
+            if (sl == SPC - 1) mma_commit(&empty[s]);
           }
-          if (!ok) break;
-          mma_commit(&empty[s]);
+          __syncwarp();
         }
-        if (!ok) break;
       }
-      if (!ok) atomicExch(abort_flag, 1);
     }
+    if (!ok && lane == 0) atomicExch(abort_flag, 1);
   } else {
     // epilogue warps
     const int wq = warp & 3, half = (warp - 2) >> 2;
