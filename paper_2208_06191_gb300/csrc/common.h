@@ -152,6 +152,7 @@ struct fem_problem {
   cbddc::DVec<int> lslot_ptr, lslot_src;
   cbddc::DVec<int> status;                  // device error bits
   cbddc::DVec<double> scratch;              // norms etc.
+  cbddc::DVec<double> hex2_geo;             // Q2: reference geometry at the Gauss points
   bool has_tangent = false;
   // autotuned setup per precision (index 0 FP64, 1 FP32): sweep block,
   // tile order (-1: not tuned yet) and the measured setup times

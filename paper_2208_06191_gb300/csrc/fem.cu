@@ -520,6 +520,200 @@ element_kernel(MatParams mp, const double* __restrict__ coords, const int* __res
 }
 
 
+// Reference geometry of the Q2 element at its 27 Gauss points, once per mesh:
+// inverse reference Jacobian (9), w detJ0 (1) and fibre frame (9), stored
+// [element][entry][point].
+constexpr int H2_GEO = 19;
+
+__global__ void hex2_geometry_kernel(MatParams mp, const double* __restrict__ coords,
+                                     const int* __restrict__ elems, const double* __restrict__ fib, int n_el,
+                                     double* __restrict__ geo) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= (int64_t)n_el * 27) return;
+  const int64_t e = t / 27;
+  const int q = (int)(t % 27), qx = q % 3, qy = (q / 3) % 3, qz = q / 9;
+  double J0[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  double Xq[3] = {0, 0, 0}, fq[3] = {0, 0, 0}, nq[3] = {0, 0, 0};
+  for (int a = 0; a < 27; ++a) {
+    const int ax = a % 3, ay = (a / 3) % 3, az = a / 9;
+    const double lx = c_L[1][qx][ax], ly = c_L[1][qy][ay], lz = c_L[1][qz][az];
+    const double dn[3] = {c_dL[1][qx][ax] * ly * lz, lx * c_dL[1][qy][ay] * lz, lx * ly * c_dL[1][qz][az]};
+    const double n = lx * ly * lz;
+    const int64_t node = elems[e * 27 + a];
+    for (int i = 0; i < 3; ++i) {
+      const double x = coords[node * 3 + i];
+      Xq[i] += n * x;
+      for (int j = 0; j < 3; ++j) J0[i][j] += x * dn[j];
+    }
+    if (mp.nodal)
+      for (int i = 0; i < 3; ++i) { fq[i] += n * fib[node * 6 + i]; nq[i] += n * fib[node * 6 + 3 + i]; }
+  }
+  double J0i[3][3], R[3][3];
+  const double det0 = inv3(J0, J0i);
+  if (mp.nodal) frame_from_fn(fq, nq, R);
+  else fibre_frame(mp, Xq, R);
+  double* g = geo + e * (H2_GEO * 27) + q;
+  for (int i = 0; i < 9; ++i) g[27 * i] = J0i[i / 3][i % 3];
+  g[27 * 9] = c_w[1][qx] * c_w[1][qy] * c_w[1][qz] * det0;
+  for (int i = 0; i < 9; ++i) g[27 * (10 + i)] = R[i / 3][i % 3];
+}
+
+// Residual of Q2 elements, one warp per element, lane = Gauss point (or node,
+// or mixed index) x + 3 (y + 3 z) of 27.  FP64 issue bounds the element
+// kernels (2 FMAs per SM and clock), so this one spends as few as it can: the
+// displacement gradient and its transpose go direction by direction (24
+// instead of 243 FMAs per component and point), the reference geometry is read
+// back (152 bytes per point) instead of formed again, and all four warps of a
+// CTA evaluate material points.  With the element kernel, whose 27 material
+// threads out of 256 also formed the geometry, the residual of 2898 elements
+// with a time state took 1348 us.
+constexpr int H2_WARPS = 4;
+
+__global__ void __launch_bounds__(32 * H2_WARPS)
+hex2_residual_kernel(MatParams mp, const int* __restrict__ elems, const double* __restrict__ geo,
+                     const double* __restrict__ d_full, const double* __restrict__ acc_full,
+                     double* __restrict__ rcontrib, int* __restrict__ status, int n_el) {
+  __shared__ double tab[2][9];                 // L, L' as [point][node]
+  __shared__ double buf[H2_WARPS][2][9 * 27];  // stage buffers
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < 9) {
+    tab[0][threadIdx.x] = c_L[1][threadIdx.x / 3][threadIdx.x % 3];
+    tab[1][threadIdx.x] = c_dL[1][threadIdx.x / 3][threadIdx.x % 3];
+  }
+  __syncthreads();
+  const int64_t e = blockIdx.x * (int64_t)H2_WARPS + warp;
+  if (e >= n_el) return;
+  const bool on = lane < 27;
+  const int l = on ? lane : 0;
+  const int x = l % 3, y = (l / 3) % 3, z = l / 9;
+  double (*b0)[27] = reinterpret_cast<double (*)[27]>(buf[warp][0]);
+  double (*b1)[27] = reinterpret_cast<double (*)[27]>(buf[warp][1]);
+  const double* L = tab[0];
+  const double* D = tab[1];
+  const int64_t node = elems[e * 27 + l];
+  // gradient with respect to the reference coordinates, and (inertia) the
+  // values of d - 2 d' + d'' at the points: stages x, y, z
+  const bool inertia = mp.rho_dt2 > 0.0;
+  if (on)
+    for (int i = 0; i < 3; ++i) b0[i][l] = d_full[node * 3 + i];
+  __syncwarp();
+  if (on)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double* u = &b0[i][3 * (y + 3 * z)];
+      b1[2 * i][l] = L[3 * x] * u[0] + L[3 * x + 1] * u[1] + L[3 * x + 2] * u[2];
+      b1[2 * i + 1][l] = D[3 * x] * u[0] + D[3 * x + 1] * u[1] + D[3 * x + 2] * u[2];
+    }
+  __syncwarp();
+  if (on)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double* v = &b1[2 * i][x + 9 * z];
+      const double* w = &b1[2 * i + 1][x + 9 * z];
+      b0[3 * i][l] = L[3 * y] * w[0] + L[3 * y + 1] * w[3] + L[3 * y + 2] * w[6];       // d/dx
+      b0[3 * i + 1][l] = D[3 * y] * v[0] + D[3 * y + 1] * v[3] + D[3 * y + 2] * v[6];   // d/dy
+      b0[3 * i + 2][l] = L[3 * y] * v[0] + L[3 * y + 1] * v[3] + L[3 * y + 2] * v[6];   // value
+    }
+  __syncwarp();
+  double F[3][3], J0i[3][3], wd;
+  {
+    const double* g = geo + e * (H2_GEO * 27) + l;
+    double R[3][3], P[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) J0i[i / 3][i % 3] = g[27 * i];
+    wd = g[27 * 9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) R[i / 3][i % 3] = g[27 * (10 + i)];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double* hx = &b0[3 * i][x + 3 * y];
+      const double* hy = &b0[3 * i + 1][x + 3 * y];
+      const double* hv = &b0[3 * i + 2][x + 3 * y];
+      const double H[3] = {L[3 * z] * hx[0] + L[3 * z + 1] * hx[9] + L[3 * z + 2] * hx[18],
+                           L[3 * z] * hy[0] + L[3 * z + 1] * hy[9] + L[3 * z + 2] * hy[18],
+                           D[3 * z] * hv[0] + D[3 * z + 1] * hv[9] + D[3 * z + 2] * hv[18]};
+#pragma unroll
+      for (int J = 0; J < 3; ++J)
+        F[i][J] = (i == J ? 1.0 : 0.0) + H[0] * J0i[0][J] + H[1] * J0i[1][J] + H[2] * J0i[2][J];
+    }
+    const bool ok = wd > 0.0 && material_point(mp, F, R, P, nullptr);
+    if (on && !ok) atomicOr(status, DEV_INVERTED);
+    // Q_ij = w detJ0 sum_J P_iJ J0i_jJ, reusing F
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        F[i][j] = ok ? wd * (P[3 * i] * J0i[j][0] + P[3 * i + 1] * J0i[j][1] + P[3 * i + 2] * J0i[j][2]) : 0.0;
+  }
+  // transposed stages z, y, x
+  __syncwarp();
+  if (on)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) b1[i][l] = F[i / 3][i % 3];
+  __syncwarp();
+  if (on)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double* q0 = &b1[3 * i][x + 3 * y];
+      const double* q1 = &b1[3 * i + 1][x + 3 * y];
+      const double* q2 = &b1[3 * i + 2][x + 3 * y];
+      b0[3 * i][l] = L[z] * q0[0] + L[3 + z] * q0[9] + L[6 + z] * q0[18];
+      b0[3 * i + 1][l] = L[z] * q1[0] + L[3 + z] * q1[9] + L[6 + z] * q1[18];
+      b0[3 * i + 2][l] = D[z] * q2[0] + D[3 + z] * q2[9] + D[6 + z] * q2[18];
+    }
+  __syncwarp();
+  if (on)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double* q0 = &b0[3 * i][x + 9 * z];
+      const double* q1 = &b0[3 * i + 1][x + 9 * z];
+      const double* q2 = &b0[3 * i + 2][x + 9 * z];
+      b1[2 * i][l] = L[y] * q0[0] + L[3 + y] * q0[3] + L[6 + y] * q0[6];
+      b1[2 * i + 1][l] = D[y] * q1[0] + D[3 + y] * q1[3] + D[6 + y] * q1[6] + L[y] * q2[0] + L[3 + y] * q2[3] +
+                         L[6 + y] * q2[6];
+    }
+  __syncwarp();
+  double r[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double* p0 = &b1[2 * i][3 * (y + 3 * z)];
+    const double* p1 = &b1[2 * i + 1][3 * (y + 3 * z)];
+    r[i] = D[x] * p0[0] + D[3 + x] * p0[1] + D[6 + x] * p0[2] + L[x] * p1[0] + L[3 + x] * p1[1] + L[6 + x] * p1[2];
+  }
+  if (inertia) {
+    // rho / dt^2 sum_q w detJ0 N_a (d - 2 d' + d'')(q)
+    double v[3];
+    __syncwarp();
+    if (on)
+      for (int i = 0; i < 3; ++i) b0[i][l] = acc_full[node * 3 + i];
+#pragma unroll
+    for (int st = 0; st < 6; ++st) {
+      // stages x, y, z to the points, then z, y, x back to the nodes
+      const int dir = st < 3 ? st : 5 - st;
+      double (*src)[27] = (st & 1) ? b1 : b0;
+      double (*dst)[27] = (st & 1) ? b0 : b1;
+      const int c = dir == 0 ? x : dir == 1 ? y : z;
+      const int at = dir == 0 ? l - x : dir == 1 ? l - 3 * y : l - 9 * z;
+      const int inc = dir == 0 ? 1 : dir == 1 ? 3 : 9;
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s += (st < 3 ? L[3 * c + k] : L[3 * k + c]) * src[i][at + inc * k];
+        v[i] = st == 2 ? wd * s : s;
+      }
+      if (on && st < 5)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) dst[i][l] = v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r[i] += mp.rho_dt2 * v[i];
+  }
+  if (on)
+    for (int i = 0; i < 3; ++i) rcontrib[(e * 27 + l) * 3 + i] = r[i];
+}
+
 // Quadrature-point-parallel element kernel for elements with few points
 // (P1: 1, P2: 4, Q1: 8; shape table O = 0, 1, 2), TET_THREADS material
 // points per CTA (EPB = TET_THREADS / NQ elements), so that every lane of
@@ -976,6 +1170,9 @@ void assemble(fem_problem* P, const double* d, double lam, double* residual, boo
       qp_element_kernel<8, 8, 2><<<grid, TET_THREADS, 0, s>>>(mp, P->coords.p, P->elems.p, fib, P->d_full.p,
                                                               accf, P->rcontrib.p, P->contrib.p, P->status.p, wt,
                                                               P->n_el);
+  } else if (!want_tangent) {
+    hex2_residual_kernel<<<cdiv(P->n_el, H2_WARPS), 32 * H2_WARPS, 0, s>>>(
+        mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, P->status.p, P->n_el);
   } else {
     element_kernel<2, 256><<<P->n_el, 256, 0, s>>>(mp, P->coords.p, P->elems.p, fib, P->d_full.p,
                                                     accf, P->rcontrib.p, P->contrib.p, P->status.p, wt);
@@ -1042,6 +1239,16 @@ void assemble(fem_problem* P, const double* d, double lam, double* residual, boo
     CB_LAUNCH();
     P->has_tangent = true;
   }
+}
+
+// Reference geometry kept with the problem (Q2 meshes).
+void prepare_geometry(fem_problem* P) {
+  if (P->tet || P->order != 2 || P->n_el == 0) return;
+  P->hex2_geo.alloc((size_t)P->n_el * H2_GEO * 27);
+  hex2_geometry_kernel<<<cdiv((int64_t)P->n_el * 27, 128), 128>>>(make_params(P, 1.0), P->coords.p, P->elems.p,
+                                                                  P->fib_nodal.p, P->n_el, P->hex2_geo.p);
+  CB_LAUNCH();
+  CB_CUDA(cudaDeviceSynchronize());
 }
 
 // y = K x, three threads per block row: thread 3 i + r forms row r of the

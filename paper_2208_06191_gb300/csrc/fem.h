@@ -14,6 +14,7 @@ void build_local_slots(fem_problem* P, const std::vector<int>& cptr, const std::
                        const std::vector<int>& cpart, const std::vector<int64_t>& cbase);
 void hex_face_node_list(int k, int f, int* out);
 void init_shape_tables(int order);
+void prepare_geometry(fem_problem* P);  // after the tables and the uploads
 
 // Element/face residual (and tangent when want_tangent) into the
 // contribution buffers, then gathers into residual (may be null) and, with

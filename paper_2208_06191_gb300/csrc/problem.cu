@@ -493,6 +493,7 @@ void build_problem(const fem_problem_desc* d, fem_problem* P) {
   CB_CUDA(cudaMemset(P->status.p, 0, P->status.bytes()));
   P->scratch.alloc(4096);
   init_shape_tables(P->order);
+  prepare_geometry(P);
 }
 
 }  // namespace cbddc
@@ -504,5 +505,5 @@ int64_t fem_problem::device_bytes() const {
                    bsr_col.bytes() + bsr_vals.bytes() + slot_ptr.bytes() + slot_src.bytes() +
                    res_ptr.bytes() + res_src.bytes() + lslot_sub.bytes() + lslot_row.bytes() +
                    lslot_col.bytes() + lslot_ptr.bytes() + lslot_src.bytes() + status.bytes() +
-                   scratch.bytes());
+                   scratch.bytes() + hex2_geo.bytes());
 }
