@@ -51,7 +51,7 @@ __device__ inline T warp_sum(T v) {
 }
 
 __device__ inline float vdot2(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
-__device__ inline double vdot2(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
+__device__ inline double vdot2(double2 a, double2 b) { return fma(a.x, b.x, a.y * b.y); }
 
 // Dot products of two rows (16-byte aligned) with a shared-memory vector,
 // one warp: the rows go in chunks of 32 x U 16-byte vectors, and every lane
@@ -95,12 +95,73 @@ __device__ __forceinline__ void warp_dot2(const T* __restrict__ ra, const T* __r
   ob = has_b ? warp_sum(acc_b) : T(0);
 }
 
+// FP64 rows, eight per warp.  The products are bound by FP64 issue (2 per SM
+// and clock: 4.8 TB/s at one FMA per entry), so no instruction is spent beside
+// the FMA of each entry: two chains per row instead of a multiplication, an
+// FMA and an addition per pair, and the eight sums of a warp are reduced
+// together, halving the number of rows at each exchange (9 additions for
+// eight rows instead of 40).  Lane 4 q holds the sum of row q at the end.
+// Rows past the last repeat it (their loads hit the cache).
+__device__ __forceinline__ double warp_dot8(const double* __restrict__ A, int64_t ld, int rows,
+                                            const double* __restrict__ xs, int n, int lane) {
+  const int nv = n / 2;
+  const double2* xv = reinterpret_cast<const double2*>(xs);
+  const double2* p[8];
+  double s0[8], s1[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    p[q] = reinterpret_cast<const double2*>(A + (int64_t)min(q, rows - 1) * ld);
+    s0[q] = s1[q] = 0.0;
+  }
+#pragma unroll 2
+  for (int i = lane; i < nv; i += 32) {
+    double2 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = __ldcs(p[q] + i);
+    const double2 x = xv[i];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      s0[q] = fma(v[q].x, x.x, s0[q]);
+      s1[q] = fma(v[q].y, x.y, s1[q]);
+    }
+  }
+  if ((n & 1) && lane == 0) {
+    const double x = xs[n - 1];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s0[q] = fma(A[(int64_t)min(q, rows - 1) * ld + n - 1], x, s0[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) s0[q] += s1[q];
+  // exchanges over 16, 8 and 4 lanes keep half of the rows each
+#pragma unroll
+  for (int w = 4; w > 0; w >>= 1) {
+    const bool up = (lane & (4 * w)) != 0;
+#pragma unroll
+    for (int q = 0; q < w; ++q) {
+      const double keep = up ? s0[q + w] : s0[q], give = up ? s0[q] : s0[q + w];
+      s0[q] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * w);
+    }
+  }
+  s0[0] += __shfl_xor_sync(0xffffffffu, s0[0], 2);
+  s0[0] += __shfl_xor_sync(0xffffffffu, s0[0], 1);
+  return s0[0];
+}
+
 // Row-block GEMV driver: rows [rb, re) of a matrix with leading dimension
-// ld, 8 warps x two rows at a time; f(row, value) stores each result.
+// ld, 8 warps x two rows at a time (FP64: eight); f(row, value) stores each
+// result.
 template <typename T, typename F>
 __device__ __forceinline__ void gemv_rows(const T* __restrict__ A, int64_t ld, int rb, int re,
                                           const T* __restrict__ xs, int n, F f) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if constexpr (sizeof(T) == 8) {
+    for (int r = rb + 8 * warp; r < re; r += 64) {
+      const int rows = min(8, re - r);
+      const double v = warp_dot8(A + (int64_t)r * ld, ld, rows, xs, n, lane);
+      if ((lane & 3) == 0 && (lane >> 2) < rows) f(r + (lane >> 2), v);
+    }
+    return;
+  }
   for (int r = rb + 2 * warp; r < re; r += 16) {
     const bool hb = (r + 1) < re;
     T va, vb;
