@@ -8,6 +8,7 @@
 // residual recomputed.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include <cooperative_groups.h>
 
@@ -23,6 +24,11 @@ namespace {
 
 constexpr int DOT_THREADS = 256;
 constexpr int64_t kCoopMaxN = 1000000;  // longest vector for the cooperative orthogonalisation
+// Longest vector whose orthogonalisation keeps a chunk of w per CTA; above, it
+// goes in tiles.  Mean Arnoldi step over 100 vectors, chunks against tiles:
+// 117 and 159 us at n = 126k, 208 and 231 us at 259k, 224 and 224 us at 304k,
+// 388 and 341 us at 608k.
+constexpr int64_t kChunkMaxN = 300000;
 constexpr int MAXV = 128;       // Krylov vectors of the cooperative orthogonalisation
 constexpr int MAXR = 1024;      // Krylov vectors per cycle (restart <= MAXR - 1)
 
@@ -174,31 +180,49 @@ __global__ void __launch_bounds__(DOT_THREADS) fused_dots_kernel(DotArgs a) {
 // Column j of the Hessenberg matrix from h1 + h2 (the two CGS passes) and
 // ||w||^2, previous rotations, the new rotation and the residual estimate.
 // scal[0] = |g_{j+1}| / ||b||, scal[1] = 1 / h_{j+1,j}, scal[2] = ||b||.
+// Run by a whole CTA: the column and the rotations come into shared memory
+// (sm: 3 (j + 1) doubles) first, because the chain over the j rotations is
+// serial, and on global memory each link cost an L2 round trip (0.35 us; 9 us
+// of a 100 us Arnoldi step at j = 25).
 __device__ void givens_update(int j, int m, double* __restrict__ H, double* __restrict__ cs,
                               double* __restrict__ sn, double* __restrict__ g, const double* h1,
                               const double* h2, double wn2, double* __restrict__ scal, double rtol,
-                              int* __restrict__ done, int* __restrict__ iters) {
-  double* col = H + (int64_t)j * (m + 1);
-  for (int i = 0; i <= j; ++i) col[i] = h2 ? h1[i] + h2[i] : h1[i];
-  const double hn = sqrt(fmax(wn2, 0.0));
-  col[j + 1] = hn;
-  scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
+                              int* __restrict__ done, int* __restrict__ iters, double* sm) {
+  double* col = sm;
+  double* c = sm + (j + 1);
+  double* s = sm + 2 * (j + 1);
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+    col[i] = h2 ? h1[i] + h2[i] : h1[i];
+    if (i < j) {
+      c[i] = cs[i];
+      s[i] = sn[i];
+    }
   }
-  const double den = hypot(col[j], col[j + 1]);
-  cs[j] = den > 0.0 ? col[j] / den : 1.0;
-  sn[j] = den > 0.0 ? col[j + 1] / den : 0.0;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  const double res = fabs(g[j + 1]) / scal[2];
-  scal[0] = res;
-  *iters += 1;
-  if (res <= rtol || hn == 0.0) *done = 1;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double hn = sqrt(fmax(wn2, 0.0));
+    scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
+    double cur = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double nxt = col[i + 1];
+      const double t = c[i] * cur + s[i] * nxt;
+      cur = -s[i] * cur + c[i] * nxt;
+      col[i] = t;
+    }
+    const double den = hypot(cur, hn);
+    cs[j] = den > 0.0 ? cur / den : 1.0;
+    sn[j] = den > 0.0 ? hn / den : 0.0;
+    col[j] = den;
+    g[j + 1] = -sn[j] * g[j];
+    g[j] = cs[j] * g[j];
+    const double res = fabs(g[j + 1]) / scal[2];
+    scal[0] = res;
+    *iters += 1;
+    if (res <= rtol || hn == 0.0) *done = 1;
+  }
+  __syncthreads();
+  double* out = H + (int64_t)j * (m + 1);
+  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) out[i] = i <= j ? col[i] : 0.0;
 }
 
 __global__ void givens_kernel(int j, int m, double* __restrict__ H, double* __restrict__ cs,
@@ -206,22 +230,39 @@ __global__ void givens_kernel(int j, int m, double* __restrict__ H, double* __re
                               const double* __restrict__ h1, const double* __restrict__ h2,
                               const double* __restrict__ wn2, double* __restrict__ scal, double rtol,
                               int* __restrict__ done, int* __restrict__ iters) {
+  __shared__ double sm[3 * MAXR];
   if (*done) return;
-  givens_update(j, m, H, cs, sn, g, h1, h2, wn2[0], scal, rtol, done, iters);
+  __syncthreads();  // every thread has read the flag
+  givens_update(j, m, H, cs, sn, g, h1, h2, wn2[0], scal, rtol, done, iters, sm);
 }
 
 // The whole orthogonalisation of one Arnoldi step in one cooperative launch
 // (all CTAs resident, grid-wide barriers): h1 = V^T w; w -= V h1, h2 = V^T w;
 // w -= V h2, ||w||^2; the Givens update (CTA 0) and v_{j+1} = w / ||w||.
-// Row tiles of 256 go to the CTAs round-robin; each warp keeps partial dot
-// products of its columns in registers across tiles, every CTA writes its
-// partials, and after each barrier every CTA sums all CTAs' partials in CTA
-// order (identical on every CTA, independent of scheduling).  This replaces
-// five launches and their tails, which dominate at small n.
+//
+// Every CTA keeps a contiguous chunk of w in shared memory through the whole
+// step.  FP64 issue is the limit (4 (j + 1) n FMAs at 2 per SM and clock), so
+// the work is spread over all SMs and all warps at any basis size and little
+// is issued beside the FMAs: dots take eight columns per warp and a segment of
+// the rows, and reduce the eight sums together at the end of the chunk (9
+// additions instead of 40); updates take 32 rows and a part of the columns per
+// warp.  The second phase goes through the chunk in tiles, update then dots,
+// so that the dots find the tile's part of V in the cache.  After each barrier
+// every CTA sums all CTAs' partials in CTA order (identical on every CTA,
+// independent of scheduling).
+// Mean Arnoldi step of a solve: 60 us at n = 86k and 59 vectors (100 us with
+// 256-row tiles dealt to half of the SMs, one column per warp and a Givens
+// chain on global memory), 51 us at n = 27k and 90 vectors (114 us).
+constexpr int CGS_THREADS = 512;
+constexpr int CGS_WARPS = CGS_THREADS / 32;
+constexpr int CGS_JS = 4;  // column parts of the update, at most
+constexpr int CGS_TILE = 32 * CGS_WARPS;  // rows of a tile (one 32-row block per warp)
 struct CgsArgs {
   const double* V;   // nvec columns of length n (stride n)
   int64_t n;
   int nvec;          // j + 1
+  int rows;          // rows per CTA
+  int js;            // column parts of the update
   double* w;
   double* vnext;     // column j + 1
   double* part;      // [3][gridDim.x][MAXV]
@@ -231,7 +272,177 @@ struct CgsArgs {
   int *done, *iters;
 };
 
-__device__ void cgs_phase(const CgsArgs& a, const double* hin, bool norm, double* ws, double* part) {
+// This warp's share of V^T ws: columns c0 .. c0 + 7 over the rows of segment
+// seg (32-row blocks seg, seg + nseg, ...); at most one share per warp.
+struct CgsDots {
+  int c0, seg, nseg;
+  bool active;
+  double s[8];
+  __device__ CgsDots(int nvec) {
+    const int warp = threadIdx.x >> 5;
+    const int ng = (nvec + 7) / 8;                    // groups of eight columns
+    nseg = max(1, CGS_WARPS / ng);                    // row segments
+    c0 = 8 * (warp % ng);
+    seg = warp / ng;
+    active = seg < nseg;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] = 0.0;
+  }
+  // rows [t0, t1) of the chunk (t0 a multiple of 32)
+  __device__ void add(const CgsArgs& a, const double* __restrict__ ws, int64_t r0, int t0, int t1) {
+    if (!active) return;
+    const int lane = threadIdx.x & 31;
+    const double* p[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) p[q] = a.V + (int64_t)min(c0 + q, a.nvec - 1) * a.n + r0;
+#pragma unroll 2
+    for (int r = t0 + 32 * seg + lane; r < t1; r += 32 * nseg) {
+      const double x = ws[r];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s[q] = fma(__ldg(p[q] + r), x, s[q]);
+    }
+  }
+  // part[0:nvec] = the CTA's sums; psum: [CGS_WARPS][MAXV] shared
+  __device__ void finish(const CgsArgs& a, double* psum, double* __restrict__ part) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (active) {
+#pragma unroll
+      for (int w = 4; w > 0; w >>= 1) {
+        const bool up = (lane & (4 * w)) != 0;
+#pragma unroll
+        for (int q = 0; q < w; ++q) {
+          const double keep = up ? s[q + w] : s[q], give = up ? s[q] : s[q + w];
+          s[q] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * w);
+        }
+      }
+      s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+      s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+      if ((lane & 3) == 0) psum[seg * MAXV + c0 + (lane >> 2)] = s[0];
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < a.nvec; c += CGS_THREADS) {
+      double t = psum[c];
+      for (int q = 1; q < nseg; ++q) t += psum[q * MAXV + c];
+      part[c] = t;
+    }
+  }
+};
+
+// ws -= V h over the rows [t0, t1) of the chunk; upd: [js][a.rows] shared (js
+// > 1).  Ends with a barrier.
+__device__ void cgs_update(const CgsArgs& a, double* __restrict__ ws, double* __restrict__ upd, int64_t r0, int t0,
+                           int t1, const double* __restrict__ h) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rb = (t1 - t0 + 31) / 32;
+  for (int it = warp; it < rb * a.js; it += CGS_WARPS) {
+    const int r = t0 + 32 * (it % rb) + lane, part = it / rb;
+    if (r < t1) {
+      const double* p = a.V + r0 + r;
+      double s = 0.0;
+#pragma unroll 8
+      for (int c = part; c < a.nvec; c += a.js) s = fma(__ldg(p + (int64_t)c * a.n), h[c], s);
+      if (a.js == 1) ws[r] -= s;
+      else upd[part * a.rows + r] = s;
+    }
+  }
+  __syncthreads();
+  if (a.js > 1) {
+    for (int r = t0 + threadIdx.x; r < t1; r += CGS_THREADS) {
+      double t = upd[r];
+      for (int q = 1; q < a.js; ++q) t += upd[q * a.rows + r];
+      ws[r] -= t;
+    }
+    __syncthreads();
+  }
+}
+
+// sums of every CTA's partials into out[0:nout] (shared memory): every warp
+// 32 columns over every WARPS-th CTA, combined in a fixed order (identical
+// on every CTA, independent of scheduling)
+template <int WARPS>
+__device__ void cgs_reduce(const double* part, int nout, double* psum, double* out) {
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  for (int j0 = 0; j0 < nout; j0 += 32) {
+    const int j = j0 + lane;
+    double s = 0.0;
+    if (j < nout) {
+#pragma unroll 4
+      for (unsigned c = grp; c < gridDim.x; c += WARPS) s += __ldcg(part + (int64_t)c * MAXV + j);
+    }
+    psum[grp * 33 + lane] = s;
+    __syncthreads();
+    if (grp == 0 && j < nout) {
+      double t = psum[lane];
+      for (int q = 1; q < WARPS; ++q) t += psum[q * 33 + lane];
+      out[j] = t;
+    }
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
+  cg::grid_group grid = cg::this_grid();
+  if (*a.done) return;  // read by every CTA before any barrier: uniform
+  extern __shared__ double cgs_smem[];
+  __shared__ double psum[CGS_WARPS * MAXV];
+  __shared__ double h1[MAXV], h2[MAXV], wn2s[1];
+  double* ws = cgs_smem;               // [a.rows]
+  double* upd = cgs_smem + a.rows;     // [js][a.rows] if js > 1
+  const int64_t r0 = (int64_t)blockIdx.x * a.rows;
+  const int rows = (int)max((int64_t)0, min((int64_t)a.rows, a.n - r0));
+  const int64_t stride = (int64_t)gridDim.x * MAXV;
+  double* part = a.part + (int64_t)blockIdx.x * MAXV;
+  for (int r = threadIdx.x; r < rows; r += CGS_THREADS) ws[r] = a.w[r0 + r];
+  __syncthreads();
+  {
+    CgsDots d(a.nvec);
+    d.add(a, ws, r0, 0, rows);
+    d.finish(a, psum, part);
+  }
+  grid.sync();
+  cgs_reduce<CGS_WARPS>(a.part, a.nvec, psum, h1);
+  {
+    CgsDots d(a.nvec);
+    const int tile = a.js > 1 ? rows : CGS_TILE;
+    for (int t0 = 0; t0 < rows; t0 += tile) {
+      const int t1 = min(rows, t0 + tile);
+      cgs_update(a, ws, upd, r0, t0, t1, h1);
+      d.add(a, ws, r0, t0, t1);
+    }
+    d.finish(a, psum, part + stride);
+  }
+  grid.sync();
+  cgs_reduce<CGS_WARPS>(a.part + stride, a.nvec, psum, h2);
+  cgs_update(a, ws, upd, r0, 0, rows, h2);
+  {
+    double s = 0.0;
+    for (int r = threadIdx.x; r < rows; r += CGS_THREADS) s = fma(ws[r], ws[r], s);
+    s = wsum(s);
+    if ((threadIdx.x & 31) == 0) psum[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = psum[0];
+      for (int q = 1; q < CGS_WARPS; ++q) t += psum[q];
+      part[2 * stride] = t;
+    }
+  }
+  grid.sync();
+  cgs_reduce<CGS_WARPS>(a.part + 2 * stride, 1, psum, wn2s);
+  if (blockIdx.x == 0)
+    givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, h1, h2, wn2s[0], a.scal, a.rtol, a.done, a.iters, psum);
+  // v_{j+1} = w / ||w|| (the same value on every CTA)
+  const double hn = sqrt(fmax(wn2s[0], 0.0));
+  const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
+  for (int r = threadIdx.x; r < rows; r += CGS_THREADS) a.vnext[r0 + r] = ws[r] * inv;
+}
+
+// The same step for vectors above kChunkMaxN unknowns, where V streams from
+// HBM: 256-row tiles dealt round-robin, w in global memory, a row per thread in
+// the updates and whole columns per warp in the dots.  Neighbouring CTAs then
+// read neighbouring tiles of the same column, which HBM serves better than the
+// chunks' 304 distant streams, and the FMAs hide behind it.
+__device__ void tiles_phase(const CgsArgs& a, const double* hin, bool norm, double* ws, double* part) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int CPW = MAXV / (DOT_THREADS / 32);  // columns per warp
   double acc[CPW];
@@ -283,41 +494,23 @@ __device__ void cgs_phase(const CgsArgs& a, const double* hin, bool norm, double
   }
 }
 
-// sums of every CTA's partials into out[0:nout] (shared memory): 4 threads
-// per output, each over every 4th CTA, combined in a fixed order (identical
-// on every CTA, independent of scheduling)
-__device__ void cgs_reduce(const double* part, int nout, double* out) {
-  __shared__ double red4[4][64];
-  const int jl = threadIdx.x & 63, grp = threadIdx.x >> 6;
-  for (int j0 = 0; j0 < nout; j0 += 64) {
-    const int j = j0 + jl;
-    double sacc = 0.0;
-    if (j < nout)
-      for (unsigned c = grp; c < gridDim.x; c += 4) sacc += __ldcg(part + (int64_t)c * MAXV + j);
-    red4[grp][jl] = sacc;
-    __syncthreads();
-    if (grp == 0 && j < nout) out[j] = (red4[0][jl] + red4[1][jl]) + (red4[2][jl] + red4[3][jl]);
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(DOT_THREADS) cgs2_coop_kernel(CgsArgs a) {
+__global__ void __launch_bounds__(DOT_THREADS) cgs2_tiles_kernel(CgsArgs a) {
   cg::grid_group grid = cg::this_grid();
   if (*a.done) return;  // read by every CTA before any barrier: uniform
-  __shared__ double ws[DOT_THREADS];
+  __shared__ double ws[DOT_THREADS], psum[DOT_THREADS / 32 * 33 > 3 * MAXV ? DOT_THREADS / 32 * 33 : 3 * MAXV];
   __shared__ double h1[MAXV], h2[MAXV], wn2s[1];
   const int64_t stride = (int64_t)gridDim.x * MAXV;
-  cgs_phase(a, nullptr, false, ws, a.part);
+  tiles_phase(a, nullptr, false, ws, a.part);
   grid.sync();
-  cgs_reduce(a.part, a.nvec, h1);
-  cgs_phase(a, h1, false, ws, a.part + stride);
+  cgs_reduce<DOT_THREADS / 32>(a.part, a.nvec, psum, h1);
+  tiles_phase(a, h1, false, ws, a.part + stride);
   grid.sync();
-  cgs_reduce(a.part + stride, a.nvec, h2);
-  cgs_phase(a, h2, true, ws, a.part + 2 * stride);
+  cgs_reduce<DOT_THREADS / 32>(a.part + stride, a.nvec, psum, h2);
+  tiles_phase(a, h2, true, ws, a.part + 2 * stride);
   grid.sync();
-  cgs_reduce(a.part + 2 * stride, 1, wn2s);
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, h1, h2, wn2s[0], a.scal, a.rtol, a.done, a.iters);
+  cgs_reduce<DOT_THREADS / 32>(a.part + 2 * stride, 1, psum, wn2s);
+  if (blockIdx.x == 0)
+    givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, h1, h2, wn2s[0], a.scal, a.rtol, a.done, a.iters, psum);
   // v_{j+1} = w / ||w|| (the same value on every CTA)
   const double hn = sqrt(fmax(wn2s[0], 0.0));
   const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
@@ -357,6 +550,7 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_coop_kernel(MgsArgs a) {
   if (*a.done) return;  // read by every CTA before any barrier: uniform
   __shared__ double red[MGS_THREADS / 32];
   __shared__ double hsh;
+  __shared__ double gsm[3 * MAXR];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = gridDim.x;
   // warp-contiguous rows: the warp's segment of 32 RPT rows, lane + 32 k
@@ -407,8 +601,9 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_coop_kernel(MgsArgs a) {
 #pragma unroll
   for (int k = 0; k < RPT; ++k) nacc = fma(x[k], x[k], nacc);
   const double wn2 = grid_sum(nacc, (a.j + 1) & 1);
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, a.hcol, nullptr, wn2, a.scal, a.rtol, a.done, a.iters);
+  // (thread 0 of CTA 0 wrote hcol; the barriers since then order it)
+  if (blockIdx.x == 0)
+    givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, a.hcol, nullptr, wn2, a.scal, a.rtol, a.done, a.iters, gsm);
   const double hn = sqrt(fmax(wn2, 0.0));
   const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
   double* op = a.vnext + base;
@@ -519,21 +714,32 @@ void Gmres::ensure_small(int64_t n_) {
 void Gmres::ensure(int64_t n_, int m_) {
   ensure_small(n_);
   if (n == n_ && m == m_) return;
-  // cooperative orthogonalisation: at most two CTAs per SM, about four row
-  // tiles per CTA; 0 when the device cannot launch cooperatively
+  // cooperative orthogonalisation; 0 when the device cannot launch
+  // cooperatively
   {
     int dev = 0, coop = 0, sms = 0, per_sm = 0;
     CB_CUDA(cudaGetDevice(&dev));
     CB_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     CB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_coop_kernel, DOT_THREADS, 0));
-    const int64_t tiles = cdiv(n_, DOT_THREADS);
-    // a few row tiles per CTA, so that the cross-CTA sums stay short; long
-    // vectors (n > 1M, bandwidth-bound) keep the multi-launch path with its
-    // larger row tiles
-    coop_grid = (coop && n_ <= kCoopMaxN) ? (int)std::min<int64_t>(std::min(per_sm, 2) * (int64_t)sms,
-                                                                   std::max<int64_t>(1, tiles / 4))
-                                          : 0;
+    coop_grid = 0;
+    cgs_rows = 0;
+    if (coop && n_ <= kChunkMaxN) {
+      // two CTAs per SM, fewer for short vectors: the FMAs shrink with the
+      // grid and the sums of its partials grow with it
+      const int64_t g = std::max<int64_t>(1, (int64_t)std::sqrt(2.0 * (double)n_));
+      coop_grid = (int)std::min<int64_t>((n_ >= 1024 * (int64_t)sms ? 2 : 1) * sms, g);
+      cgs_rows = (int)round_up(cdiv(n_, coop_grid), 32);
+      coop_grid = (int)cdiv(n_, cgs_rows);
+      cgs_js = (int)std::min<int64_t>(CGS_JS, std::max<int64_t>(1, 4 * CGS_WARPS / (cgs_rows / 32)));
+      cgs_smem = (size_t)cgs_rows * (cgs_js > 1 ? 1 + cgs_js : 1) * sizeof(double);
+      CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_coop_kernel, CGS_THREADS, cgs_smem));
+      if (coop_grid > per_sm * sms) coop_grid = cgs_rows = 0;
+    }
+    if (coop && n_ <= kCoopMaxN && coop_grid == 0) {
+      CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_tiles_kernel, DOT_THREADS, 0));
+      coop_grid = (int)std::min<int64_t>(std::min(per_sm, 2) * (int64_t)sms,
+                                         std::max<int64_t>(1, cdiv(n_, DOT_THREADS) / 4));
+    }
     if (coop_grid > 0) cpart.alloc((size_t)3 * coop_grid * MAXV);
     // MGS cooperative launch: one CTA of MGS_THREADS per SM, rows per
     // thread rounded up to 8, 16, 24 or 32 (n up to 3.1M on 152 SMs; 0:
@@ -656,11 +862,13 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
       timer_begin(CBDDC_TIMER_ORTH, s);
       if (G.coop_grid > 0 && j + 1 <= MAXV) {
         // short vectors and bases: CGS2 in one cooperative launch
-        CgsArgs ca{G.V.p, n, j + 1, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.cpart.p, j, m,
+        CgsArgs ca{G.V.p, n, j + 1, G.cgs_rows, G.cgs_js, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.cpart.p, j, m,
                    G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
         void* args[] = {&ca};
-        CB_CUDA(cudaLaunchCooperativeKernel((const void*)cgs2_coop_kernel, dim3(G.coop_grid),
-                                            dim3(DOT_THREADS), args, 0, s));
+        const bool chunks = G.cgs_rows > 0;
+        CB_CUDA(cudaLaunchCooperativeKernel(chunks ? (const void*)cgs2_coop_kernel : (const void*)cgs2_tiles_kernel,
+                                            dim3(G.coop_grid), dim3(chunks ? CGS_THREADS : DOT_THREADS), args,
+                                            chunks ? G.cgs_smem : 0, s));
         CB_LAUNCH();
       } else if (G.mgs_grid > 0) {
         MgsArgs ma{G.V.p, n, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.mpart.p, G.h.p, j, m,
@@ -685,7 +893,7 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
         CB_LAUNCH();
         fused_dots(G, G.V.p, n, j + 1, G.w.p, n, nullptr, 0, h2, done, s, reorth);
         fused_dots(G, G.V.p, n, j + 1, G.w.p, n, h2, 1, wn2, done, s, reorth);
-        givens_kernel<<<1, 1, 0, s>>>(j, m, G.H.p, G.cs.p, G.sn.p, G.g.p, h1, h2, wn2, G.scal.p, rtol,
+        givens_kernel<<<1, 256, 0, s>>>(j, m, G.H.p, G.cs.p, G.sn.p, G.g.p, h1, h2, wn2, G.scal.p, rtol,
                                       done, kcount);
         CB_LAUNCH();
         scale_kernel<<<nb, 256, 0, s>>>(G.w.p, G.V.p + (int64_t)(j + 1) * n, n, G.scal.p, 1, done);
