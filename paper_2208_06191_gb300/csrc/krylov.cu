@@ -704,11 +704,11 @@ void Gmres::ensure_small(int64_t n_) {
   CB_CUDA(cudaMemset(ticket.p, 0, sizeof(unsigned)));
   hstride = MAXV;
   h.alloc(3 * hstride);
-  scal.alloc(8);
-  flags.alloc(4);
-  CB_CUDA(cudaMemset(flags.p, 0, 4 * sizeof(int)));
-  if (!host_scal) CB_CUDA(cudaMallocHost(&host_scal, 64));
-  if (!host_flags) CB_CUDA(cudaMallocHost(&host_flags, 16));
+  scal.alloc(10);
+  CB_CUDA(cudaMemset(scal.p, 0, scal.bytes()));
+  if (!host_scal) CB_CUDA(cudaMallocHost(&host_scal, 32 * sizeof(double)));
+  for (auto& e : step_done)
+    if (!e) CB_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
 }
 
 void Gmres::ensure(int64_t n_, int m_) {
@@ -787,7 +787,8 @@ void Gmres::ensure(int64_t n_, int m_) {
 
 Gmres::~Gmres() {
   if (host_scal) cudaFreeHost(host_scal);
-  if (host_flags) cudaFreeHost(host_flags);
+  for (auto& e : step_done)
+    if (e) cudaEventDestroy(e);
 }
 
 // out = V^T w over nvec columns (stride ldv), optionally after w -= V hin,
@@ -819,14 +820,75 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
   G.ensure(n, restart);
   const int m = restart;
   const unsigned nb = cdiv(n, 256);
-  int* done = G.flags.p;
-  int* kcount = G.flags.p + 1;
+  int* done = G.flags();
+  int* kcount = G.flags() + 1;
   CB_CUDA(cudaMemsetAsync(x, 0, n * sizeof(double), s));
   int total = 0;
   bool first = true;
-  int* hflags = G.host_flags;
-  CB_CUDA(cudaMemsetAsync(G.flags.p + 3, 0, sizeof(int), s));  // second Gram-Schmidt passes
+  CB_CUDA(cudaMemsetAsync(G.flags() + 3, 0, sizeof(int), s));  // second Gram-Schmidt passes
   bool converged = false;
+  int flags[4] = {0, 0, 0, 0};  // the device's, as last read
+  // scalars and flags of the device into a pinned slot
+  auto fetch = [&](int slot) {
+    CB_CUDA(cudaMemcpyAsync(G.host_scal + 10 * slot, G.scal.p, 10 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CB_CUDA(cudaEventRecord(G.step_done[slot], s));
+  };
+  // Arnoldi step j of a cycle: v_j -> z_j = M^-1 v_j, w = K z_j, and w made
+  // orthonormal to the basis
+  auto arnoldi_step = [&](int j) {
+    double* vj = G.V.p + (int64_t)j * n;
+    double* zj = G.Zb.p + (int64_t)j * n;
+    bddc_run_apply(C, vj, zj, s);
+    bsr_spmv(P, zj, G.w.p, s);
+    double* h1 = G.h.p;
+    double* h2 = G.h.p + G.hstride;
+    double* wn2 = G.h.p + 2 * G.hstride;
+    timer_begin(CBDDC_TIMER_ORTH, s);
+    if (G.coop_grid > 0 && j + 1 <= MAXV) {
+      // short vectors and bases: CGS2 in one cooperative launch
+      CgsArgs ca{G.V.p, n, j + 1, G.cgs_rows, G.cgs_js, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.cpart.p, j, m,
+                 G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
+      void* args[] = {&ca};
+      const bool chunks = G.cgs_rows > 0;
+      CB_CUDA(cudaLaunchCooperativeKernel(chunks ? (const void*)cgs2_coop_kernel : (const void*)cgs2_tiles_kernel,
+                                          dim3(G.coop_grid), dim3(chunks ? CGS_THREADS : DOT_THREADS), args,
+                                          chunks ? G.cgs_smem : 0, s));
+      CB_LAUNCH();
+    } else if (G.mgs_grid > 0) {
+      MgsArgs ma{G.V.p, n, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.mpart.p, G.h.p, j, m,
+                 G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
+      void* args[] = {&ma};
+      const void* fn = G.mgs_rpt == 8    ? (const void*)mgs_coop_kernel<8>
+                       : G.mgs_rpt == 16 ? (const void*)mgs_coop_kernel<16>
+                       : G.mgs_rpt == 24 ? (const void*)mgs_coop_kernel<24>
+                                         : (const void*)mgs_coop_kernel<32>;
+      CB_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G.mgs_grid), dim3(MGS_THREADS), args, 0, s));
+      CB_LAUNCH();
+    } else {
+      // classical Gram-Schmidt with a second pass only where the first
+      // one lost more than half of ||w||^2 (Daniel-Gragg-Kaufman-Stewart
+      // criterion, eta = 1/sqrt(2)): h1 = V^T w with ||w||^2; w -= V h1
+      // with the new ||w||^2; then, gated on the device, h2 = V^T w and
+      // w -= V h2 with its norm
+      int* reorth = G.flags() + 2;
+      fused_dots(G, G.V.p, n, j + 1, G.w.p, n, nullptr, 0, h1, done, s, nullptr, 1);
+      fused_dots(G, G.V.p, n, j + 1, G.w.p, n, h1, 1, wn2, done, s);
+      dgks_kernel<<<1, 256, 0, s>>>(h1, j + 1, wn2, h2, reorth, G.flags() + 3, done);
+      CB_LAUNCH();
+      fused_dots(G, G.V.p, n, j + 1, G.w.p, n, nullptr, 0, h2, done, s, reorth);
+      fused_dots(G, G.V.p, n, j + 1, G.w.p, n, h2, 1, wn2, done, s, reorth);
+      givens_kernel<<<1, 256, 0, s>>>(j, m, G.H.p, G.cs.p, G.sn.p, G.g.p, h1, h2, wn2, G.scal.p, rtol, done,
+                                      kcount);
+      CB_LAUNCH();
+      scale_kernel<<<nb, 256, 0, s>>>(G.w.p, G.V.p + (int64_t)(j + 1) * n, n, G.scal.p, 1, done);
+      CB_LAUNCH();
+    }
+    // algorithmic traffic of one Gram-Schmidt pass (the second pass, when
+    // taken, is not counted): V read twice (dots, update), w read twice
+    // and written once, v_{j+1} written
+    timer_end(CBDDC_TIMER_ORTH, s, 4.0 * (j + 1) * (double)n, 8.0 * (double)n * (2.0 * (j + 1) + 4.0));
+    fetch(j & 1);
+  };
   while (true) {
     // r = b - K x
     if (first) {
@@ -841,103 +903,62 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
     CB_LAUNCH();
     scale_kernel<<<nb, 256, 0, s>>>(G.r.p, G.V.p, n, G.scal.p, 1, nullptr);
     CB_LAUNCH();
-    CB_CUDA(cudaMemcpyAsync(G.host_scal, G.scal.p, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CB_CUDA(cudaMemcpyAsync(hflags, done, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    fetch(0);
     CB_CUDA(cudaStreamSynchronize(s));
     first = false;
-    *relres_out = G.host_scal[0];
-    if (hflags[0]) { converged = true; break; }
+    std::memcpy(flags, G.host_scal + 8, sizeof flags);
+    double res = G.host_scal[0];  // residual estimate of the last step known here
+    *relres_out = res;
+    if (flags[0]) { converged = true; break; }
     if (total >= max_iters) break;
-    int j = 0;
-    for (; j < m && total < max_iters; ++j) {
-      double* vj = G.V.p + (int64_t)j * n;
-      double* zj = G.Zb.p + (int64_t)j * n;
-      bddc_run_apply(C, vj, zj, s);
-      bsr_spmv(P, zj, G.w.p, s);
-      // classical Gram-Schmidt, twice: h1 = V^T w; w -= V h1 and h2 = V^T w;
-      // w -= V h2 and ||w||^2 (three launches)
-      double* h1 = G.h.p;
-      double* h2 = G.h.p + G.hstride;
-      double* wn2 = G.h.p + 2 * G.hstride;
-      timer_begin(CBDDC_TIMER_ORTH, s);
-      if (G.coop_grid > 0 && j + 1 <= MAXV) {
-        // short vectors and bases: CGS2 in one cooperative launch
-        CgsArgs ca{G.V.p, n, j + 1, G.cgs_rows, G.cgs_js, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.cpart.p, j, m,
-                   G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
-        void* args[] = {&ca};
-        const bool chunks = G.cgs_rows > 0;
-        CB_CUDA(cudaLaunchCooperativeKernel(chunks ? (const void*)cgs2_coop_kernel : (const void*)cgs2_tiles_kernel,
-                                            dim3(G.coop_grid), dim3(chunks ? CGS_THREADS : DOT_THREADS), args,
-                                            chunks ? G.cgs_smem : 0, s));
-        CB_LAUNCH();
-      } else if (G.mgs_grid > 0) {
-        MgsArgs ma{G.V.p, n, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.mpart.p, G.h.p, j, m,
-                   G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
-        void* args[] = {&ma};
-        const void* fn = G.mgs_rpt == 8    ? (const void*)mgs_coop_kernel<8>
-                         : G.mgs_rpt == 16 ? (const void*)mgs_coop_kernel<16>
-                         : G.mgs_rpt == 24 ? (const void*)mgs_coop_kernel<24>
-                                           : (const void*)mgs_coop_kernel<32>;
-        CB_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G.mgs_grid), dim3(MGS_THREADS), args, 0, s));
-        CB_LAUNCH();
-      } else {
-        // classical Gram-Schmidt with a second pass only where the first
-        // one lost more than half of ||w||^2 (Daniel-Gragg-Kaufman-Stewart
-        // criterion, eta = 1/sqrt(2)): h1 = V^T w with ||w||^2; w -= V h1
-        // with the new ||w||^2; then, gated on the device, h2 = V^T w and
-        // w -= V h2 with its norm
-        int* reorth = G.flags.p + 2;
-        fused_dots(G, G.V.p, n, j + 1, G.w.p, n, nullptr, 0, h1, done, s, nullptr, 1);
-        fused_dots(G, G.V.p, n, j + 1, G.w.p, n, h1, 1, wn2, done, s);
-        dgks_kernel<<<1, 256, 0, s>>>(h1, j + 1, wn2, h2, reorth, G.flags.p + 3, done);
-        CB_LAUNCH();
-        fused_dots(G, G.V.p, n, j + 1, G.w.p, n, nullptr, 0, h2, done, s, reorth);
-        fused_dots(G, G.V.p, n, j + 1, G.w.p, n, h2, 1, wn2, done, s, reorth);
-        givens_kernel<<<1, 256, 0, s>>>(j, m, G.H.p, G.cs.p, G.sn.p, G.g.p, h1, h2, wn2, G.scal.p, rtol,
-                                      done, kcount);
-        CB_LAUNCH();
-        scale_kernel<<<nb, 256, 0, s>>>(G.w.p, G.V.p + (int64_t)(j + 1) * n, n, G.scal.p, 1, done);
-        CB_LAUNCH();
-      }
-      // algorithmic traffic of one Gram-Schmidt pass (the second pass, when
-      // taken, is not counted): V read twice (dots, update), w read twice
-      // and written once, v_{j+1} written
-      timer_end(CBDDC_TIMER_ORTH, s, 4.0 * (j + 1) * (double)n, 8.0 * (double)n * (2.0 * (j + 1) + 4.0));
-      CB_CUDA(cudaMemcpyAsync(hflags, done, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
-      CB_CUDA(cudaStreamSynchronize(s));
+    // The host reads the residual of every step.  Waiting for it before the
+    // next step is launched left the GPU idle for the copy, the wake-up and the
+    // first launches (25-55 us of each 200-350 us step on the smaller meshes),
+    // so one further step is launched before step j's residual is known,
+    // unless that residual can be expected to end the solve (one step gains
+    // less than a factor of five): a step launched too many is skipped by the
+    // Gram-Schmidt kernels, at the price of its apply and product.
+    const int steps = std::min(m, max_iters - total);
+    int launched = 0;
+    for (int j = 0; j < steps; ++j) {
+      while (launched < steps && (launched <= j || (launched == j + 1 && res > 5.0 * rtol))) arnoldi_step(launched++);
+      CB_CUDA(cudaEventSynchronize(G.step_done[j & 1]));
+      const double* slot = G.host_scal + 10 * (j & 1);
+      std::memcpy(flags, slot + 8, sizeof flags);
+      res = slot[0];
       ++total;
-      if (hflags[0]) { ++j; break; }
+      if (flags[0]) break;
     }
     // x += Z y over the columns built in this cycle
     backsolve_kernel<<<1, 256, 0, s>>>(G.H.p, m, kcount, G.g.p, G.y.p);
     CB_LAUNCH();
     combine_kernel<<<nb, 256, 0, s>>>(G.Zb.p, n, kcount, G.y.p, x, n);
     CB_LAUNCH();
-    if (total >= max_iters && !hflags[0]) {
+    if (total >= max_iters && !flags[0]) {
       // final true residual
       bsr_spmv(P, x, G.w.p, s);
       axpby_kernel<<<nb, 256, 0, s>>>(1.0, b, -1.0, G.w.p, G.r.p, n);
       CB_LAUNCH();
       fused_dots(G, G.r.p, n, 1, G.r.p, n, nullptr, 1, G.h.p, nullptr, s);
-      CB_CUDA(cudaMemcpyAsync(G.host_scal + 4, G.h.p, sizeof(double), cudaMemcpyDeviceToHost, s));
+      CB_CUDA(cudaMemcpyAsync(G.host_scal + 20, G.h.p, sizeof(double), cudaMemcpyDeviceToHost, s));
       CB_CUDA(cudaMemcpyAsync(G.host_scal, G.scal.p, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
       CB_CUDA(cudaStreamSynchronize(s));
-      *relres_out = G.host_scal[2] > 0 ? std::sqrt(G.host_scal[4]) / G.host_scal[2] : 0.0;
+      *relres_out = G.host_scal[2] > 0 ? std::sqrt(G.host_scal[20]) / G.host_scal[2] : 0.0;
       break;
     }
     // next cycle (or final check) recomputes the true residual
   }
   *iters_out = total;
-  G.reorth = hflags[3];
+  G.reorth = flags[3];
   return converged ? CBDDC_OK : CBDDC_ENOCONV;
 }
 
 double device_norm(fem_problem* P, Gmres& G, const double* v, cudaStream_t s) {
   G.ensure_small(P->n_free);
   fused_dots(G, v, P->n_free, 1, const_cast<double*>(v), P->n_free, nullptr, 1, G.h.p, nullptr, s);
-  CB_CUDA(cudaMemcpyAsync(G.host_scal + 4, G.h.p, sizeof(double), cudaMemcpyDeviceToHost, s));
+  CB_CUDA(cudaMemcpyAsync(G.host_scal + 20, G.h.p, sizeof(double), cudaMemcpyDeviceToHost, s));
   CB_CUDA(cudaStreamSynchronize(s));
-  return std::sqrt(G.host_scal[4]);
+  return std::sqrt(G.host_scal[20]);
 }
 
 void axpby(double a, const double* x, double b, const double* y, double* out, int64_t n, cudaStream_t s) {

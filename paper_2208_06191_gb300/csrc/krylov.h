@@ -14,7 +14,9 @@ struct Gmres {
   int hstride = 0;           // stride of the three CGS coefficient vectors in h
   int reorth = 0;            // second Gram-Schmidt passes of the last solve
   DVec<double> V, Zb, w, r, H, cs, sn, g, y, h, partial, scal;
-  DVec<int> flags;
+  // {done, Krylov vectors, second pass, second passes} live behind the eight
+  // scalars, so that one copy per Arnoldi step brings both to the host
+  int* flags() const { return reinterpret_cast<int*>(scal.p + 8); }
   DVec<unsigned> ticket;
   DVec<double> cpart;        // per-CTA partials of the cooperative orthogonalisation
   int coop_grid = 0;         // its grid size (0: use the multi-launch path)
@@ -22,8 +24,8 @@ struct Gmres {
   size_t cgs_smem = 0;
   DVec<double> mpart;        // per-CTA partials of the cooperative MGS step
   int mgs_grid = 0, mgs_rpt = 0;  // its grid and rows per thread (0: not available)
-  double* host_scal = nullptr;
-  int* host_flags = nullptr;
+  double* host_scal = nullptr;  // pinned: two slots of 10 doubles, then a spare
+  cudaEvent_t step_done[2] = {nullptr, nullptr};  // copies of the slots
   void ensure_small(int64_t n_);
   void ensure(int64_t n_, int m_);
   Gmres() = default;
