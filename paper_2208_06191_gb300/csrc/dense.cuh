@@ -755,19 +755,24 @@ sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat
 }
 
 // Builds X and Y panels and zeroes the pivot rows/columns, for indices
-// [blockIdx.x*PANEL_CH, +PANEL_CH) of each matrix (as columns for Y, as rows
-// for X).  Reads and writes of different CTAs touch disjoint entries: the Y
-// part reads pivot rows outside the pivot columns, the X part reads pivot
-// columns outside the pivot rows (the pivot block itself is read only into
-// Y entries that are replaced by P).  Narrow chunks keep many CTAs in flight
-// (a single coarse matrix still spreads over the GPU); each thread forms
-// NB / 16 rows of one Y column and gathers its NB / 16 X entries before
-// storing.  Shared memory (dynamic): P (NB x NB+1) and the chunk of pivot
-// rows (NB x CH+1).
-constexpr int PANEL_CH = 16;
-template <typename T, int NB>
+// [blockIdx.x*CH, +CH) of each matrix (as columns for Y, as rows for X).
+// Reads and writes of different CTAs touch disjoint entries: the Y part reads
+// pivot rows outside the pivot columns, the X part reads pivot columns outside
+// the pivot rows (the pivot block itself is read only into Y entries that are
+// replaced by P).  256 threads as 16 x 16; each forms NB / 16 rows of CH / 16
+// columns of Y.  Shared memory (dynamic): P (NB x NB+1) and the chunk of pivot
+// rows (NB x CH+4).
+//
+// Chunks of 64 read P once per 64 indices and give every P and pivot-row entry
+// read from shared memory four uses; with chunks of 16, P (16 to 64 KB) was
+// most of what a CTA read.  FP32, 64-wide blocks: 41 us per step against 50 us
+// (48x48x12 slab), 121 us against 163 us (P2 ventricle, 582k unknowns).  Lists too
+// short to fill the GPU with chunks of 64 (a single coarse matrix) keep 16, and
+// so does FP64, which is bound by the FMAs of Y at 2 per SM and clock and ran
+// slower in fewer, larger CTAs (262 us with 16, 359 us with 64, same slab).
+template <typename T, int NB, int CH>
 constexpr size_t panel_smem_bytes() {
-  return sizeof(T) * ((size_t)NB * (NB + 1) + (size_t)NB * (PANEL_CH + 1));
+  return sizeof(T) * ((size_t)NB * (NB + 1) + (size_t)NB * (CH + 4));
 }
 
 //
@@ -776,17 +781,17 @@ constexpr size_t panel_smem_bytes() {
 // NB) at Xbuf, Xlo (, Xlo2) and Y^T parts (columns x NB) at Ybuf, Ylo (,
 // Ylo2), with zeros beyond the kb pivots of a partial last block, so the
 // update needs no separate split pass.
-template <typename T, int NB, int NP>
+template <typename T, int NB, int NP, int CH>
 __global__ void __launch_bounds__(256)
 sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat,
                    const T* __restrict__ Pbuf, T* __restrict__ Xbuf, T* __restrict__ Ybuf,
                    T* __restrict__ Xlo, T* __restrict__ Ylo, T* __restrict__ Xlo2, T* __restrict__ Ylo2) {
   constexpr bool SPLIT = NP > 0;
-  constexpr int CH = PANEL_CH, PER = NB * CH / 256, RY = NB / 16;
-  static_assert(CH == 16 && NB % 16 == 0, "NB / 16 rows of one column per thread");
+  constexpr int PER = NB * CH / 256, RY = NB / 16, CY = CH / 16, LDC = CH + 4;
+  static_assert(NB % 16 == 0 && CH % 16 == 0, "16 x 16 threads");
   extern __shared__ __align__(16) unsigned char panel_smem[];
   T (*Ps)[NB + 1] = reinterpret_cast<T (*)[NB + 1]>(panel_smem);
-  T (*col)[CH + 1] = reinterpret_cast<T (*)[CH + 1]>(panel_smem + sizeof(T) * NB * (NB + 1));
+  T (*col)[LDC] = reinterpret_cast<T (*)[LDC]>(panel_smem + sizeof(T) * NB * (NB + 1));
   const SweepDesc d = desc[blockIdx.y];
   const int k0 = k * NB;
   if (k0 >= d.p) return;
@@ -801,11 +806,13 @@ sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ ma
   T* X = Xbuf + d.offX;
   T* Y = Ybuf + d.offY;
   if (cn > 0) {
+#pragma unroll 8
     for (int t = tid; t < NB * NB; t += 256) {
       const int r = t / NB, q = t % NB;
       Ps[r][q] = (r < kb && q < kb) ? P[r * NB + q] : T(0);
     }
     // pivot rows restricted to this column chunk (zero outside kb x cn)
+#pragma unroll 8
     for (int t = tid; t < NB * CH; t += 256) {
       const int r = t / CH, cc = t % CH;
       col[r][cc] = (r < kb && cc < cn) ? A[(int64_t)(k0 + r) * d.ld + c0 + cc] : T(0);
@@ -813,65 +820,82 @@ sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ ma
   }
   // X[i, :] = A[i, kk] (i outside kk), X[kk] = -I ; then A[i, kk] = 0
   if (rn > 0) {
-    T xv[PER];
+    constexpr int XB = PER < 16 ? PER : 16;  // entries in flight per thread
+#pragma unroll 1
+    for (int u0 = 0; u0 < PER; u0 += XB) {
+      T xv[XB];
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int t = tid + 256 * u, r = t / NB, q = t % NB, i = c0 + r;
-      xv[u] = (r < rn && q < kb && !(i >= k0 && i < k0 + kb)) ? A[(int64_t)i * d.ld + k0 + q] : T(0);
-    }
+      for (int u = 0; u < XB; ++u) {
+        const int t = tid + 256 * (u0 + u), r = t / NB, q = t % NB, i = c0 + r;
+        xv[u] = (r < rn && q < kb && !(i >= k0 && i < k0 + kb)) ? A[(int64_t)i * d.ld + k0 + q] : T(0);
+      }
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int t = tid + 256 * u, r = t / NB, q = t % NB, i = c0 + r;
-      if (SPLIT) {
-        if (r < rn) {
+      for (int u = 0; u < XB; ++u) {
+        const int t = tid + 256 * (u0 + u), r = t / NB, q = t % NB, i = c0 + r;
+        if (SPLIT) {
+          if (r < rn) {
+            const bool piv = i >= k0 && i < k0 + kb;
+            const T x = q < kb ? (piv ? ((i - k0 == q) ? T(-1) : T(0)) : xv[u]) : T(0);
+            float parts[3];
+            tc::split_tf32<NP == 3 ? 3 : 2>((float)x, parts);
+            X[(int64_t)i * NB + q] = parts[0];
+            Xlo[d.offX + (int64_t)i * NB + q] = parts[1];
+            if (NP == 3) Xlo2[d.offX + (int64_t)i * NB + q] = parts[2];
+            if (q < kb) A[(int64_t)i * d.ld + k0 + q] = T(0);
+          }
+        } else if (r < rn && q < kb) {
           const bool piv = i >= k0 && i < k0 + kb;
-          const T x = q < kb ? (piv ? ((i - k0 == q) ? T(-1) : T(0)) : xv[u]) : T(0);
-          float parts[3];
-          tc::split_tf32<NP == 3 ? 3 : 2>((float)x, parts);
-          X[(int64_t)i * NB + q] = parts[0];
-          Xlo[d.offX + (int64_t)i * NB + q] = parts[1];
-          if (NP == 3) Xlo2[d.offX + (int64_t)i * NB + q] = parts[2];
-          if (q < kb) A[(int64_t)i * d.ld + k0 + q] = T(0);
+          X[(int64_t)i * NB + q] = piv ? ((i - k0 == q) ? T(-1) : T(0)) : xv[u];
+          A[(int64_t)i * d.ld + k0 + q] = T(0);
         }
-      } else if (r < rn && q < kb) {
-        const bool piv = i >= k0 && i < k0 + kb;
-        X[(int64_t)i * NB + q] = piv ? ((i - k0 == q) ? T(-1) : T(0)) : xv[u];
-        A[(int64_t)i * d.ld + k0 + q] = T(0);
       }
     }
   }
   if (cn == 0) return;
   __syncthreads();
   // Y[r, j] = sum_q P[r][q] A[k0+q, j]  (j outside kk),  Y[:, kk] = P
-  const int ty = tid / CH, c = tid % CH;   // rows RY ty .. RY ty + RY - 1 of column c
-  T acc[RY];
+  const int ty = tid / 16, tx = tid % 16;  // rows RY ty .., columns tx + 16 x
+  T acc[RY][CY];
 #pragma unroll
-  for (int i = 0; i < RY; ++i) acc[i] = T(0);
+  for (int i = 0; i < RY; ++i)
+#pragma unroll
+    for (int x = 0; x < CY; ++x) acc[i][x] = T(0);
+#pragma unroll 4
   for (int q = 0; q < kb; ++q) {
-    const T cq = col[q][c];
+    T cq[CY];
 #pragma unroll
-    for (int i = 0; i < RY; ++i) acc[i] = fma(Ps[RY * ty + i][q], cq, acc[i]);
-  }
-  if (c >= cn) return;
-  const int jg = c0 + c;
-  const bool pivc = jg >= k0 && jg < k0 + kb;
+    for (int x = 0; x < CY; ++x) cq[x] = col[q][tx + 16 * x];
 #pragma unroll
-  for (int i = 0; i < RY; ++i) {
-    const int r = RY * ty + i;
-    if (SPLIT) {
-      // Y^T row jg, K index r (zero beyond kb)
-      const T y = r < kb ? (pivc ? Ps[r][jg - k0] : acc[i]) : T(0);
-      float parts[3];
-      tc::split_tf32<NP == 3 ? 3 : 2>((float)y, parts);
-      Y[(int64_t)jg * NB + r] = parts[0];
-      Ylo[d.offY + (int64_t)jg * NB + r] = parts[1];
-      if (NP == 3) Ylo2[d.offY + (int64_t)jg * NB + r] = parts[2];
-      if (r < kb) A[(int64_t)(k0 + r) * d.ld + jg] = T(0);
-      continue;
+    for (int i = 0; i < RY; ++i) {
+      const T pq = Ps[RY * ty + i][q];
+#pragma unroll
+      for (int x = 0; x < CY; ++x) acc[i][x] = fma(pq, cq[x], acc[i][x]);
     }
-    if (r >= kb) continue;
-    Y[(int64_t)r * d.ld + jg] = pivc ? Ps[r][jg - k0] : acc[i];
-    A[(int64_t)(k0 + r) * d.ld + jg] = T(0);
+  }
+#pragma unroll
+  for (int x = 0; x < CY; ++x) {
+    const int c = tx + 16 * x;
+    if (c >= cn) continue;
+    const int jg = c0 + c;
+    const bool pivc = jg >= k0 && jg < k0 + kb;
+#pragma unroll
+    for (int i = 0; i < RY; ++i) {
+      const int r = RY * ty + i;
+      if (SPLIT) {
+        // Y^T row jg, K index r (zero beyond kb)
+        const T y = r < kb ? (pivc ? Ps[r][jg - k0] : acc[i][x]) : T(0);
+        float parts[3];
+        tc::split_tf32<NP == 3 ? 3 : 2>((float)y, parts);
+        Y[(int64_t)jg * NB + r] = parts[0];
+        Ylo[d.offY + (int64_t)jg * NB + r] = parts[1];
+        if (NP == 3) Ylo2[d.offY + (int64_t)jg * NB + r] = parts[2];
+        if (r < kb) A[(int64_t)(k0 + r) * d.ld + jg] = T(0);
+        continue;
+      }
+      if (r >= kb) continue;
+      Y[(int64_t)r * d.ld + jg] = pivc ? Ps[r][jg - k0] : acc[i][x];
+      A[(int64_t)(k0 + r) * d.ld + jg] = T(0);
+    }
   }
 }
 
