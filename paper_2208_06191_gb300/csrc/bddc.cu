@@ -26,6 +26,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "bddc.h"
 #include "fem.h"
@@ -527,36 +528,96 @@ apply_interior_kernel(const int2* __restrict__ items, const int* __restrict__ nI
 // interface nodes, x: the packed interior solution) and t_I = r_I -
 // K_I,Gamma z (rows: packed interior nodes, x: z on the interface nodes).
 // One lane per block row, all nine products in the operator precision.
+//
+// S warps share a slice (S consecutive parts of its steps, added in order).
+// With a few hundred slices (slabs, small ventricles) one warp per slice leaves
+// two or three warps on an SM, and the chain of up to 125 steps is the time: S
+// = 4 below eight slices per SM (FP32, 24x24x6 Q2 slab: 62 us to 20 us; 48x48x12
+// Q1 slab: 17 us to 8 us).  Larger meshes fill the GPU with one warp per slice,
+// where more parts only add the sums at the end (there the batches of four
+// steps give 43 us to 33 us, 582k unknowns of P2).
 template <typename T> struct Q4;
 template <> struct Q4<float> { using type = float4; };
 template <> struct Q4<double> { using type = double4_32a; };
 
-template <typename T>
+template <typename T, int S>
 __global__ void __launch_bounds__(256)
 coupling_kernel(const int* __restrict__ off, const int* __restrict__ len, const int* __restrict__ rowmap,
                 const int* __restrict__ col, const T* __restrict__ val,
                 const typename Q4<T>::type* __restrict__ xq, const int* __restrict__ rdof,
                 const double* __restrict__ r, double* __restrict__ out, int nslices) {
-  const int q = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  const int q = w / S, part = w % S;
   const int lane = threadIdx.x & 31;
-  if (q >= nslices) return;
-  const int row = rowmap[32 * q + lane];
-  const int L = len[q];
-  const int64_t base = off[q];
+  if (S == 1 && q >= nslices) return;
+  const bool in = q < nslices;
+  const int L = in ? len[q] : 0;
+  const int64_t base = in ? off[q] : 0;
   T a0 = T(0), a1 = T(0), a2 = T(0);
-#pragma unroll 2
-  for (int k = 0; k < L; ++k) {
-    const typename Q4<T>::type x = xq[__ldg(col + (base + k) * 32 + lane)];
-    const T* v = val + (base + k) * 288 + lane;
-    a0 = fma(__ldcs(v + 0), x.x, fma(__ldcs(v + 32), x.y, fma(__ldcs(v + 64), x.z, a0)));
-    a1 = fma(__ldcs(v + 96), x.x, fma(__ldcs(v + 128), x.y, fma(__ldcs(v + 160), x.z, a1)));
-    a2 = fma(__ldcs(v + 192), x.x, fma(__ldcs(v + 224), x.y, fma(__ldcs(v + 256), x.z, a2)));
+  // Batches of U steps: their columns, then their inputs and values, then the
+  // sums in step order, so that U steps are in flight.
+  int k = L * part / S;
+  const int k1 = L * (part + 1) / S;
+  auto batch = [&](auto size) {
+    constexpr int U = decltype(size)::value;
+    for (; k + U <= k1; k += U) {
+      int c[U];
+      typename Q4<T>::type x[U];
+      T v[U][9];
+#pragma unroll
+      for (int u = 0; u < U; ++u) c[u] = __ldg(col + (base + k + u) * 32 + lane);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        x[u] = xq[c[u]];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) v[u][e] = __ldcs(val + (base + k + u) * 288 + 32 * e + lane);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a0 = fma(v[u][0], x[u].x, fma(v[u][1], x[u].y, fma(v[u][2], x[u].z, a0)));
+        a1 = fma(v[u][3], x[u].x, fma(v[u][4], x[u].y, fma(v[u][5], x[u].z, a1)));
+        a2 = fma(v[u][6], x[u].x, fma(v[u][7], x[u].y, fma(v[u][8], x[u].z, a2)));
+      }
+    }
+  };
+  batch(std::integral_constant<int, 4>());
+  batch(std::integral_constant<int, 2>());
+  batch(std::integral_constant<int, 1>());
+  if constexpr (S > 1) {
+    __shared__ T sums[256 / 32][3][32];
+    const int wl = threadIdx.x >> 5;
+    sums[wl][0][lane] = a0;
+    sums[wl][1][lane] = a1;
+    sums[wl][2][lane] = a2;
+    __syncthreads();
+    if (part != 0 || !in) return;
+#pragma unroll
+    for (int p = 1; p < S; ++p) {
+      a0 += sums[wl + p][0][lane];
+      a1 += sums[wl + p][1][lane];
+      a2 += sums[wl + p][2][lane];
+    }
   }
+  const int row = rowmap[32 * q + lane];
   if (row >= 0) {
     out[3 * (int64_t)row + 0] = r[rdof[3 * row + 0]] - (double)a0;
     out[3 * (int64_t)row + 1] = r[rdof[3 * row + 1]] - (double)a1;
     out[3 * (int64_t)row + 2] = r[rdof[3 * row + 2]] - (double)a2;
   }
+}
+
+template <typename T>
+void launch_coupling(int nslices, cudaStream_t s, const int* off, const int* len, const int* rowmap, const int* col,
+                     const T* val, const void* xq, const int* rdof, const double* r, double* out) {
+  if (nslices == 0) return;
+  const auto* x = static_cast<const typename Q4<T>::type*>(xq);
+  if (nslices < 8 * 152)
+    coupling_kernel<T, 4><<<cdiv((int64_t)nslices * 4 * 32, 256), 256, 0, s>>>(off, len, rowmap, col, val, x, rdof,
+                                                                              r, out, nslices);
+  else
+    coupling_kernel<T, 1><<<cdiv((int64_t)nslices * 32, 256), 256, 0, s>>>(off, len, rowmap, col, val, x, rdof, r,
+                                                                          out, nslices);
+  CB_LAUNCH();
 }
 
 // Values of the sliced coupling blocks from the assembled tangent, in the
@@ -1914,14 +1975,13 @@ void apply_with_work(bddc_ctx* C, const double* r, double* z, const ApplyWork& w
   }
   if (C->n_if > 0) {
     if (C->sparse_cpl) {  // g = r_Gamma - K_Gamma,I u0
-      coupling_kernel<T><<<cdiv((int64_t)C->n_sgi * 32, 256), 256, 0, s>>>(
-          C->sgi_off.p, C->sgi_len.p, C->sgi_row.p, C->sgi_col.p, reinterpret_cast<const T*>(C->sgi_val.p),
-          static_cast<const typename Q4<T>::type*>(w.uq), C->if_dof.p, r, w.gI, C->n_sgi);
+      launch_coupling<T>(C->n_sgi, s, C->sgi_off.p, C->sgi_len.p, C->sgi_row.p, C->sgi_col.p,
+                         reinterpret_cast<const T*>(C->sgi_val.p), w.uq, C->if_dof.p, r, w.gI);
     } else {
       assemble_g_kernel<<<cdiv(C->n_if, 256), 256, 0, s>>>(C->if_dof.p, C->if_ptr.p, C->if_src.p, C->n_if,
                                                           r, w.hG, w.gI);
+      CB_LAUNCH();
     }
-    CB_LAUNCH();
     restrict_kernel<<<cdiv(C->totG, 256), 256, 0, s>>>(C->gam_if.p, C->Dg.p, C->totG, w.gI, w.gl);
     CB_LAUNCH();
     if (C->n_dlx > 0) {  // deluxe: g_i = D_b^T g on each class
@@ -1986,10 +2046,8 @@ void apply_with_work(bddc_ctx* C, const double* r, double* z, const ApplyWork& w
   if (C->sparse_cpl) {
     // z_I = A_II^-1 (r_I - K_I,Gamma z): the coupling overwrites the
     // gathered r_I (no longer needed) with its right-hand side
-    coupling_kernel<T><<<cdiv((int64_t)C->n_sig * 32, 256), 256, 0, s>>>(
-        C->sig_off.p, C->sig_len.p, C->sig_row.p, C->sig_col.p, reinterpret_cast<const T*>(C->sig_val.p),
-        static_cast<const typename Q4<T>::type*>(w.zq), C->gdofI.p, r, w.xI, C->n_sig);
-    CB_LAUNCH();
+    launch_coupling<T>(C->n_sig, s, C->sig_off.p, C->sig_len.p, C->sig_row.p, C->sig_col.p,
+                       reinterpret_cast<const T*>(C->sig_val.p), w.zq, C->gdofI.p, r, w.xI);
     apply_interior_kernel<T, true><<<C->n_itI, 256, smI, s>>>(
         C->itI.p, C->d_nI.p, C->d_offA.p, C->d_ldA.p, C->d_offI.p, C->gdofI.p, Aloc, w.xI, z, nullptr);
     CB_LAUNCH();
