@@ -767,17 +767,36 @@ apply_phit_kernel(const int2* __restrict__ items, const int* __restrict__ nG, co
 }
 
 // rc[p] = sum over the listed local primal entries of all their chunks
-// (cnch[q]: chunks of the subdomain that owns local entry q).
+// (cnch[q]: chunks of the subdomain that owns local entry q), in order.  A few
+// hundred threads: bound by the latency of source -> chunk count -> chunks, so
+// four sources' indices and eight chunks are loaded together.
 __global__ void coarse_rhs_kernel(const int* __restrict__ ptr, const int* __restrict__ src, int n,
                                   const double* __restrict__ clp, int nchunk,
                                   const int* __restrict__ cnch, double* __restrict__ rc) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
+  const int j1 = ptr[m + 1];
   double v = 0.0;
-  for (int j = ptr[m]; j < ptr[m + 1]; ++j) {
-    const double* q = clp + (int64_t)src[j] * nchunk;
-    const int nc = cnch[src[j]];
-    for (int c = 0; c < nc; ++c) v += q[c];
+  for (int j0 = ptr[m]; j0 < j1; j0 += 4) {
+    // (past the last source or chunk, the last one is read again)
+    int sc[4], nc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sc[u] = src[min(j0 + u, j1 - 1)];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) nc[u] = cnch[sc[u]];
+    double q[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) q[u][c] = clp[(int64_t)sc[u] * nchunk + max(0, min(c, nc[u] - 1))];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (j0 + u >= j1) break;
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (c < nc[u]) v += q[u][c];
+      for (int c = 8; c < nc[u]; ++c) v += clp[(int64_t)sc[u] * nchunk + c];
+    }
   }
   rc[m] = v;
 }
@@ -2005,7 +2024,7 @@ void apply_with_work(bddc_ctx* C, const double* r, double* z, const ApplyWork& w
                                                             w.gl, w.cl, nch);
         CB_LAUNCH();
       }
-      coarse_rhs_kernel<<<cdiv(C->n_pi, 256), 256, 0, s>>>(C->cg_ptr.p, C->cg_src.p, C->n_pi, w.cl, nch,
+      coarse_rhs_kernel<<<cdiv(C->n_pi, 64), 64, 0, s>>>(C->cg_ptr.p, C->cg_src.p, C->n_pi, w.cl, nch,
                                                            C->cnch.p, w.rc);
       CB_LAUNCH();
       if (C->next) {
