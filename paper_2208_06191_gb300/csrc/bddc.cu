@@ -1036,6 +1036,9 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
   CB_CHECK(opt != nullptr, CBDDC_EINVAL, "null options");
   CB_CHECK(opt->precision == CBDDC_FP64 || opt->precision == CBDDC_FP32, CBDDC_EINVAL, "bad precision");
   C->P = P;
+  CB_CUDA(cudaStreamCreateWithFlags(&C->side, cudaStreamNonBlocking));
+  CB_CUDA(cudaEventCreateWithFlags(&C->ev_fork, cudaEventDisableTiming));
+  CB_CUDA(cudaEventCreateWithFlags(&C->ev_join, cudaEventDisableTiming));
   C->precision = opt->precision;
   C->primal = opt->primal;
   C->pivot_tol = opt->pivot_tol > 0 ? opt->pivot_tol : 1e-13;
@@ -2009,38 +2012,54 @@ void apply_with_work(bddc_ctx* C, const double* r, double* z, const ApplyWork& w
           C->gam_if.p, reinterpret_cast<const T*>(C->Ddb.p), w.gI, w.gl);
       CB_LAUNCH();
     }
-    if (C->n_itG > 0) {
-      apply_local_kernel<T><<<C->n_itG, 256,
-                              (size_t)round_up(std::max(C->maxR, 4), 4) * sizeof(T), s>>>(
-          C->itG.p, C->d_nG.p, C->d_nr.p, C->d_offS.p, C->d_ldS.p, C->d_offGam.p, Sw, w.gl, w.wG);
-      CB_LAUNCH();
+    // The coarse correction (Phi^T g, the coarse solve) and the local solves
+    // T g are independent until the prolongation.  The coarse chain is short
+    // kernels that leave the GPU mostly idle (48x48x12 slab: 33 us beside the
+    // 46 us of T g; three levels: the whole level-2 apply), so it runs on the
+    // context's second stream between two events of the caller's.
+    const bool fork = C->n_pi > 0 && C->n_itG > 0;
+    cudaStream_t sc = s;
+    if (fork) {
+      sc = C->side;
+      CB_CUDA(cudaEventRecord(C->ev_fork, s));
+      CB_CUDA(cudaStreamWaitEvent(sc, C->ev_fork, 0));
     }
     if (C->n_pi > 0) {
       const int nch = (int)cdiv(C->maxG, PHIT_ROWS);
       if (C->n_itP > 0) {
-        apply_phit_kernel<T><<<C->n_itP, 256, 0, s>>>(C->itP.p, C->d_nG.p, C->d_nc.p, C->d_offPhi.p,
+        apply_phit_kernel<T><<<C->n_itP, 256, 0, sc>>>(C->itP.p, C->d_nG.p, C->d_nc.p, C->d_offPhi.p,
                                                             C->d_ldPhi.p, C->d_offGam.p, C->d_offC.p,
                                                             C->coarse == CBDDC_COARSE_PETROV ? Psi : Phi,
                                                             w.gl, w.cl, nch);
         CB_LAUNCH();
       }
-      coarse_rhs_kernel<<<cdiv(C->n_pi, 64), 64, 0, s>>>(C->cg_ptr.p, C->cg_src.p, C->n_pi, w.cl, nch,
+      coarse_rhs_kernel<<<cdiv(C->n_pi, 64), 64, 0, sc>>>(C->cg_ptr.p, C->cg_src.p, C->n_pi, w.cl, nch,
                                                            C->cnch.p, w.rc);
       CB_LAUNCH();
       if (C->next) {
         // the level-2 context uses its own work vectors, allocated at setup;
         // its apply is not timed on its own (an enclosing bddc_run_apply
         // times the whole recursion, and bddc_apply_noalloc times nothing)
-        timer_begin(CBDDC_TIMER_LEVEL2_APPLY, s);
-        apply_untimed(C->next.get(), w.rc, w.uc, s);
-        timer_end(CBDDC_TIMER_LEVEL2_APPLY, s, C->next->apply_flops, (double)C->next->local_bytes);
+        timer_begin(CBDDC_TIMER_LEVEL2_APPLY, sc);
+        apply_untimed(C->next.get(), w.rc, w.uc, sc);
+        timer_end(CBDDC_TIMER_LEVEL2_APPLY, sc, C->next->apply_flops, (double)C->next->local_bytes);
       } else {
-        timer_begin(CBDDC_TIMER_COARSE_APPLY, s);
-        dense_gemv_kernel<<<cdiv((int64_t)C->n_pi * 32, 256), 256, 0, s>>>(C->Sc.p, C->n_pi, w.rc, w.uc);
+        timer_begin(CBDDC_TIMER_COARSE_APPLY, sc);
+        dense_gemv_kernel<<<cdiv((int64_t)C->n_pi * 32, 256), 256, 0, sc>>>(C->Sc.p, C->n_pi, w.rc, w.uc);
         CB_LAUNCH();
-        timer_end(CBDDC_TIMER_COARSE_APPLY, s, 2.0 * (double)C->n_pi * C->n_pi,
+        timer_end(CBDDC_TIMER_COARSE_APPLY, sc, 2.0 * (double)C->n_pi * C->n_pi,
                   8.0 * (double)C->n_pi * C->n_pi);
       }
+    }
+    if (C->n_itG > 0) {
+      apply_local_kernel<T><<<C->n_itG, 256,
+                              (size_t)round_up(std::max(C->maxR, 4), 4) * sizeof(T), s>>>(
+          C->itG.p, C->d_nG.p, C->d_nr.p, C->d_offS.p, C->d_ldS.p, C->d_offGam.p, Sw, w.gl, w.wG);
+      CB_LAUNCH();
+    }
+    if (fork) {
+      CB_CUDA(cudaEventRecord(C->ev_join, sc));
+      CB_CUDA(cudaStreamWaitEvent(s, C->ev_join, 0));
     }
     if (C->n_itR > 0) {
       apply_prolong_kernel<T><<<C->n_itR, 256, 0, s>>>(
@@ -2177,6 +2196,12 @@ void bddc_run_apply_noalloc(bddc_ctx* C, const double* r, double* z, cudaStream_
 }
 
 }  // namespace cbddc
+
+bddc_ctx::~bddc_ctx() {
+  if (ev_fork) cudaEventDestroy(ev_fork);
+  if (ev_join) cudaEventDestroy(ev_join);
+  if (side) cudaStreamDestroy(side);
+}
 
 int64_t bddc_ctx::device_bytes() const {
   return (int64_t)(Aloc.bytes() + Sw.bytes() + Phi.bytes() + Y.bytes() + Zf.bytes() + Wf.bytes() +

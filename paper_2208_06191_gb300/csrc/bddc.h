@@ -99,6 +99,13 @@ struct bddc_ctx {
   std::unique_ptr<fem_problem> coarse_prob;
   std::unique_ptr<bddc_ctx> next;
   cbddc::DVec<int64_t> d_cbase;  // first coarse contribution block of each subdomain
+  // second stream of the apply (coarse correction beside the local solves)
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  bddc_ctx() = default;
+  bddc_ctx(const bddc_ctx&) = delete;
+  bddc_ctx& operator=(const bddc_ctx&) = delete;
+  ~bddc_ctx();
   int64_t device_bytes() const;
 };
 
