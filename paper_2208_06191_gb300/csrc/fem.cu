@@ -1278,11 +1278,43 @@ bsr_spmv_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
   y[t] = a0 + a1 + a2;
 }
 
+// The same product for long rows (Q2: up to 125 blocks), one warp per block
+// row: lanes 0..26 take three consecutive blocks at a time, entry (r, k) =
+// lane % 9, so a step reads 216 consecutive bytes; with three threads per row
+// every load of a warp touched eleven rows' lines and the L1 wavefronts were
+// the time.  The nine lanes of a row r are summed at the end (two shuffle
+// additions over k, three over the blocks), which short rows cannot afford:
+// taken from 40 blocks per row on average.  24x24x6 Q2 slab (57 per row):
+// 53 us against 75 us.
+__global__ void __launch_bounds__(256)
+bsr_spmv_long_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, const double* __restrict__ vals,
+                     const double* __restrict__ x, double* __restrict__ y, int nrows) {
+  const int row = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row >= nrows) return;
+  const int b0 = __ldg(row_ptr + row), b1 = __ldg(row_ptr + row + 1);
+  const int sub = lane / 9, e = lane - 9 * sub, k = e % 3;
+  double a = 0.0;
+  if (lane < 27) {
+#pragma unroll 4
+    for (int b = b0 + sub; b < b1; b += 3)
+      a = fma(__ldg(vals + (int64_t)b * 9 + e), __ldg(x + (int64_t)__ldg(col + b) * 3 + k), a);
+  }
+  // lane r (r = 0, 1, 2): sum over k and the three blocks of entry row r
+  double s = 0.0;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) s += __shfl_sync(0xffffffffu, a, 9 * (q / 3) + 3 * (lane % 3) + q % 3);
+  if (lane < 3) y[3 * (int64_t)row + lane] = s;
+}
+
 void bsr_spmv(const fem_problem* P, const double* x, double* y, cudaStream_t s) {
   const int64_t rows = P->n_free_nodes;
   timer_begin(CBDDC_TIMER_SPMV, s);
-  bsr_spmv_kernel<<<cdiv(rows * 3, 256), 256, 0, s>>>(P->bsr_row_ptr.p, P->bsr_col.p,
-                                                      P->bsr_vals.p, x, y, (int)rows);
+  if (P->nnzb >= 40 * rows)
+    bsr_spmv_long_kernel<<<cdiv(rows * 32, 256), 256, 0, s>>>(P->bsr_row_ptr.p, P->bsr_col.p, P->bsr_vals.p, x, y,
+                                                             (int)rows);
+  else
+    bsr_spmv_kernel<<<cdiv(rows * 3, 256), 256, 0, s>>>(P->bsr_row_ptr.p, P->bsr_col.p, P->bsr_vals.p, x, y,
+                                                        (int)rows);
   CB_LAUNCH();
   // bytes: 9 values + 1 column index per block, x read and y written once
   timer_end(CBDDC_TIMER_SPMV, s, 18.0 * P->nnzb, 76.0 * P->nnzb + 16.0 * 3 * rows);
