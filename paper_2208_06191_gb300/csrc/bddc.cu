@@ -476,6 +476,14 @@ __global__ void coarse_assemble_kernel_d(const int* __restrict__ key, const int*
 
 // ------------------------------------------------------------ apply kernels
 constexpr int AROWS = 128;  // rows per CTA of the prolongation (8 warps x 4 rows, 4 passes)
+// Columns of an FP64 sweep list from which Y = P A_kk is formed by the
+// tensor-core GEMM (two split launches and a GEMM) instead of FP64 FMAs in the
+// panel kernel.  Per step, FMA panel against GEMM and remaining panel: 20 us
+// against about 25 us on one to three thousand columns, where the launches cost
+// more than the FMAs; 67 us and 34 us (12 subdomains of 13k unknowns), 110 us and
+// 55 us (512 subdomains of the 27k-unknown ventricle), 312 us and 97 us (48x48x12
+// slab, 60k columns).
+constexpr int64_t kPanelColumns = 4096;
 constexpr int PHIT_ROWS = 128;  // interface rows per CTA of the coarse restriction
 constexpr int NC_MAX = 512;  // primal constraints per subdomain
 
@@ -1348,13 +1356,20 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
     out.clear();
     out.resize(steps);
     for (int k = 0; k < steps; ++k) {
-      std::vector<GemmProb> g;
+      std::vector<GemmProb> g, y;
+      int64_t cols = 0;
       for (int s = 0; s < nmat; ++s) {
         const SweepDesc& d = sw[s];
         const int kb = std::max(0, std::min(NB, d.p - k * NB));
         g.push_back(GemmProb{d.rows, d.cols, kb, NB, d.ld, d.ld, d.offX, d.offY, d.off});
+        y.push_back(GemmProb{kb, d.cols, kb, NB, d.ld, d.ld, d.offP, d.off + (int64_t)k * NB * d.ld, d.offY});
+        if (kb > 0) cols += d.cols;
       }
       out[k].set(g, es, false, to);
+      if (es == 8 && cols >= kPanelColumns) {
+        out[k].panel.reset(new GemmList);
+        out[k].panel->set(y, es, false, to);
+      }
     }
   };
   sweep_gemms(sw1, C->steps1, C->gl_sw1);
@@ -1670,7 +1685,10 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
                       &C->gl_dlx})
         lists.push_back(g);
       for (auto* v : {&C->gl_sw1, &C->gl_sw2, &C->gl_swg, &C->gl_swd})
-        for (auto& g : *v) lists.push_back(&g);
+        for (auto& g : *v) {
+          lists.push_back(&g);
+          if (g.panel) lists.push_back(g.panel.get());
+        }
     }
     int64_t need = 0;
     for (auto* g : lists) need = std::max(need, g->oz_bytes());
@@ -1731,7 +1749,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
 template <typename T, int NB, int NP, int CH>
 static void panel_launch_ch(int n, int nmat, cudaStream_t s, const SweepDesc* desc, int k, T* mat, const T* Pbuf,
                             T* X, T* Y, T* const* lo) {
-  constexpr size_t smem = panel_smem_bytes<T, NB, CH>();
+  constexpr size_t smem = NP < 0 ? 0 : panel_smem_bytes<T, NB, CH>();
   static bool attr = false;
   if (!attr) {
     CB_CUDA(cudaFuncSetAttribute(sweep_panel_kernel<T, NB, NP, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1773,7 +1791,16 @@ static void run_sweep_nb(const DVec<SweepDesc>& desc, int nmat, const std::vecto
     CB_LAUNCH();
     const int n = std::max(maxRows, maxCols);
     const bool split = sizeof(T) == 4 && lists[k].presplit && lists[k].tc_bound && tensor_cores_for(true);
-    if (split && lists[k].np == 3)
+    bool formed = false;
+    if constexpr (sizeof(T) == 8) {
+      formed = lists[k].panel && lists[k].panel->oz_base;
+      if (formed) {
+        launch_list<T, false, false>(*lists[k].panel, Pbuf, mat, Y, T(1), T(0), s);
+        panel_launch_ch<T, NB, -1, 64>(n, nmat, s, desc.p, k, mat, Pbuf, X, Y, none);
+      }
+    }
+    if (formed) {
+    } else if (split && lists[k].np == 3)
       panel_launch<T, NB, 3>(n, nmat, s, desc.p, k, mat, Pbuf, X, Y, lo);
     else if (split)
       panel_launch<T, NB, 2>(n, nmat, s, desc.p, k, mat, Pbuf, X, Y, lo);

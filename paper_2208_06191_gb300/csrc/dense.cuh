@@ -15,6 +15,7 @@
 // which is the rank-kb form of the sweep.  No pivoting: a pivot below
 // tol * max|diag| (or non-finite) sets DEV_PIVOT in the status word.
 #pragma once
+#include <memory>
 #include <algorithm>
 #include <vector>
 
@@ -326,6 +327,7 @@ struct GemmList {
   std::vector<oz::Batch> oz_batches;
   unsigned char* oz_base = nullptr;
   int* oz_status = nullptr;
+  std::unique_ptr<GemmList> panel;  // FP64 sweep step: Y = P A_kk as products of their own
   // order 1: tiles of the largest problems (M N K) first, so that with
   // uneven subdomains the long tile runs of a persistent kernel start early
   void set(const std::vector<GemmProb>& v, size_t esize, bool ta = false, int order = 0) {
@@ -781,12 +783,15 @@ constexpr size_t panel_smem_bytes() {
 // NB) at Xbuf, Xlo (, Xlo2) and Y^T parts (columns x NB) at Ybuf, Ylo (,
 // Ylo2), with zeros beyond the kb pivots of a partial last block, so the
 // update needs no separate split pass.
+//
+// NP < 0: Y's columns outside the pivots are already there (formed from the
+// untouched pivot rows by a GEMM); the rest as above, without shared memory.
 template <typename T, int NB, int NP, int CH>
 __global__ void __launch_bounds__(256)
 sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat,
                    const T* __restrict__ Pbuf, T* __restrict__ Xbuf, T* __restrict__ Ybuf,
                    T* __restrict__ Xlo, T* __restrict__ Ylo, T* __restrict__ Xlo2, T* __restrict__ Ylo2) {
-  constexpr bool SPLIT = NP > 0;
+  constexpr bool SPLIT = NP > 0, FORMED = NP < 0;
   constexpr int PER = NB * CH / 256, RY = NB / 16, CY = CH / 16, LDC = CH + 4;
   static_assert(NB % 16 == 0 && CH % 16 == 0, "16 x 16 threads");
   extern __shared__ __align__(16) unsigned char panel_smem[];
@@ -805,7 +810,7 @@ sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ ma
   const T* P = Pbuf + d.offP;
   T* X = Xbuf + d.offX;
   T* Y = Ybuf + d.offY;
-  if (cn > 0) {
+  if (!FORMED && cn > 0) {
 #pragma unroll 8
     for (int t = tid; t < NB * NB; t += 256) {
       const int r = t / NB, q = t % NB;
@@ -852,6 +857,15 @@ sweep_panel_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ ma
     }
   }
   if (cn == 0) return;
+  if constexpr (FORMED) {
+    for (int t = tid; t < kb * CH; t += 256) {
+      const int r = t / CH, c = t % CH, jg = c0 + c;
+      if (c >= cn) continue;
+      if (jg >= k0 && jg < k0 + kb) Y[(int64_t)r * d.ld + jg] = P[r * NB + jg - k0];
+      A[(int64_t)(k0 + r) * d.ld + jg] = T(0);
+    }
+    return;
+  }
   __syncthreads();
   // Y[r, j] = sum_q P[r][q] A[k0+q, j]  (j outside kk),  Y[:, kk] = P
   const int ty = tid / 16, tx = tid % 16;  // rows RY ty .., columns tx + 16 x
