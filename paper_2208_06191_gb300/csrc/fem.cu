@@ -371,155 +371,6 @@ __global__ void scatter_free_kernel(const double* __restrict__ d, const int* __r
   d_full[node * 3 + i % 3] = d[i];
 }
 
-// One CTA per element.  Order K hexahedron: M = K+1 points per direction,
-// NEN = M^3 nodes and NQ = M^3 Gauss points.
-template <int K, int THREADS>
-__global__ void __launch_bounds__(THREADS)
-element_kernel(MatParams mp, const double* __restrict__ coords, const int* __restrict__ elems,
-               const double* __restrict__ fib, const double* __restrict__ d_full,
-               const double* __restrict__ acc_full, double* __restrict__ rcontrib,
-               double* __restrict__ contrib, int* __restrict__ status, int want_tangent) {
-  constexpr int M = K + 1, NEN = M * M * M, NQ = NEN;
-  constexpr int O = K - 1;
-  __shared__ double X[NEN][3], U[NEN][3];
-  __shared__ double G[NQ][NEN][3];
-  __shared__ double Wd[NQ];
-  __shared__ double Pq[NQ][9];
-  __shared__ double Aq[NQ][81];
-  __shared__ double T[NEN * 27];
-  __shared__ double Nq[NQ][NEN], Aq3[NQ][3];  // shape values; d - 2d' + d'' at the points
-  __shared__ int bad;
-  const bool inertia = mp.rho_dt2 > 0.0;
-  const int e = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (tid == 0) bad = 0;
-  for (int t = tid; t < NEN * 3; t += THREADS) {
-    int a = t / 3, c = t % 3;
-    int node = elems[(int64_t)e * NEN + a];
-    X[a][c] = coords[(int64_t)node * 3 + c];
-    U[a][c] = d_full[(int64_t)node * 3 + c];
-  }
-  __syncthreads();
-  // geometry and constitutive update at each Gauss point
-  for (int q = tid; q < NQ; q += THREADS) {
-    const int qx = q % M, qy = (q / M) % M, qz = q / (M * M);
-    double J0[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    double Xq[3] = {0, 0, 0}, fq[3] = {0, 0, 0}, nq[3] = {0, 0, 0};
-    for (int a = 0; a < NEN; ++a) {
-      const int ax = a % M, ay = (a / M) % M, az = a / (M * M);
-      const double lx = c_L[O][qx][ax], ly = c_L[O][qy][ay], lz = c_L[O][qz][az];
-      const double dn[3] = {c_dL[O][qx][ax] * ly * lz, lx * c_dL[O][qy][ay] * lz,
-                            lx * ly * c_dL[O][qz][az]};
-      const double n = lx * ly * lz;
-      Nq[q][a] = n;
-      for (int i = 0; i < 3; ++i) {
-        Xq[i] += n * X[a][i];
-        for (int j = 0; j < 3; ++j) J0[i][j] += X[a][i] * dn[j];
-      }
-      if (mp.nodal) {
-        const double* fa = fib + (int64_t)elems[(int64_t)e * NEN + a] * 6;
-        for (int i = 0; i < 3; ++i) { fq[i] += n * fa[i]; nq[i] += n * fa[3 + i]; }
-      }
-      G[q][a][0] = dn[0];
-      G[q][a][1] = dn[1];
-      G[q][a][2] = dn[2];
-    }
-    if (inertia) {
-      double aq[3] = {0, 0, 0};
-      for (int a = 0; a < NEN; ++a) {
-        const double* va = acc_full + (int64_t)elems[(int64_t)e * NEN + a] * 3;
-        for (int i = 0; i < 3; ++i) aq[i] += Nq[q][a] * va[i];
-      }
-      for (int i = 0; i < 3; ++i) Aq3[q][i] = aq[i];
-    }
-    double J0i[3][3];
-    const double det0 = inv3(J0, J0i);
-    Wd[q] = c_w[O][qx] * c_w[O][qy] * c_w[O][qz] * det0;
-    double F[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
-    for (int a = 0; a < NEN; ++a) {
-      double dn[3] = {G[q][a][0], G[q][a][1], G[q][a][2]};
-      double gx[3];
-      for (int i = 0; i < 3; ++i) gx[i] = dn[0] * J0i[0][i] + dn[1] * J0i[1][i] + dn[2] * J0i[2][i];
-      G[q][a][0] = gx[0];
-      G[q][a][1] = gx[1];
-      G[q][a][2] = gx[2];
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) F[i][j] += U[a][i] * gx[j];
-    }
-    double R[3][3];
-    if (mp.nodal) frame_from_fn(fq, nq, R);
-    else fibre_frame(mp, Xq, R);
-    if (!(det0 > 0.0) || !material_point(mp, F, R, Pq[q], want_tangent ? Aq[q] : nullptr)) {
-      bad = 1;
-      for (int i = 0; i < 9; ++i) Pq[q][i] = 0.0;
-      if (want_tangent)
-        for (int i = 0; i < 81; ++i) Aq[q][i] = 0.0;
-    }
-  }
-  __syncthreads();
-  if (tid == 0 && bad) atomicOr(status, DEV_INVERTED);
-  // residual r_a,i = sum_q w detJ0 P_iJ dN_a/dX_J
-  for (int t = tid; t < NEN * 3; t += THREADS) {
-    const int a = t / 3, i = t % 3;
-    double r = 0.0;
-    for (int q = 0; q < NQ; ++q)
-      r += Wd[q] * (Pq[q][i * 3 + 0] * G[q][a][0] + Pq[q][i * 3 + 1] * G[q][a][1] +
-                    Pq[q][i * 3 + 2] * G[q][a][2]);
-    if (inertia)
-      for (int q = 0; q < NQ; ++q) r += mp.rho_dt2 * Wd[q] * Nq[q][a] * Aq3[q][i];
-    rcontrib[((int64_t)e * NEN + a) * 3 + i] = r;
-  }
-  if (!want_tangent) return;
-  // K[a][b][i][k] = sum_q w detJ0 sum_JL dN_a/dX_J A_iJkL dN_b/dX_L
-  constexpr int NE = NEN * NEN * 9;
-  constexpr int PER = (NE + THREADS - 1) / THREADS;
-  double acc[PER];
-#pragma unroll
-  for (int j = 0; j < PER; ++j) acc[j] = 0.0;
-  for (int q = 0; q < NQ; ++q) {
-    __syncthreads();
-    // T[a][i][k][L] = w detJ0 sum_J dN_a/dX_J A_iJkL
-    for (int t = tid; t < NEN * 27; t += THREADS) {
-      const int a = t / 27, r = t % 27, i = r / 9, k = (r / 3) % 3, L = r % 3;
-      const double* Aqq = Aq[q];
-      T[t] = Wd[q] * (G[q][a][0] * Aqq[((i * 3 + 0) * 3 + k) * 3 + L] +
-                      G[q][a][1] * Aqq[((i * 3 + 1) * 3 + k) * 3 + L] +
-                      G[q][a][2] * Aqq[((i * 3 + 2) * 3 + k) * 3 + L]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int t = tid + j * THREADS;
-      if (t < NE) {
-        const int a = t / (NEN * 9), b = (t / 9) % NEN, i = (t % 9) / 3, k = t % 3;
-        const double* Ta = &T[a * 27 + i * 9 + k * 3];
-        acc[j] += Ta[0] * G[q][b][0] + Ta[1] * G[q][b][1] + Ta[2] * G[q][b][2];
-      }
-    }
-  }
-  if (inertia) {
-    // consistent mass rho/dt^2 sum_q w detJ0 N_a N_b on the diagonal i = k
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int t = tid + j * THREADS;
-      if (t < NE) {
-        const int a = t / (NEN * 9), b = (t / 9) % NEN, i = (t % 9) / 3, k = t % 3;
-        if (i == k) {
-          double m = 0.0;
-          for (int q = 0; q < NQ; ++q) m += Wd[q] * Nq[q][a] * Nq[q][b];
-          acc[j] += mp.rho_dt2 * m;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < PER; ++j) {
-    const int t = tid + j * THREADS;
-    if (t < NE) contrib[(int64_t)e * NE + t] = acc[j];
-  }
-}
-
-
 // Reference geometry of the Q2 element at its 27 Gauss points, once per mesh:
 // inverse reference Jacobian (9), w detJ0 (1) and fibre frame (9), stored
 // [element][entry][point].
@@ -558,36 +409,57 @@ __global__ void hex2_geometry_kernel(MatParams mp, const double* __restrict__ co
   for (int i = 0; i < 9; ++i) g[27 * (10 + i)] = R[i / 3][i % 3];
 }
 
-// Residual of Q2 elements, one warp per element, lane = Gauss point (or node,
-// or mixed index) x + 3 (y + 3 z) of 27.  FP64 issue bounds the element
-// kernels (2 FMAs per SM and clock), so this one spends as few as it can: the
-// displacement gradient and its transpose go direction by direction (24
-// instead of 243 FMAs per component and point), the reference geometry is read
-// back (152 bytes per point) instead of formed again, and all four warps of a
-// CTA evaluate material points.  With the element kernel, whose 27 material
-// threads out of 256 also formed the geometry, the residual of 2898 elements
-// with a time state took 1348 us.
-constexpr int H2_WARPS = 4;
+// Q2 elements, one warp per element, lane = Gauss point (or node, or mixed
+// index) x + 3 (y + 3 z) of 27.  FP64 issue bounds the element kernels (2 FMAs
+// per SM and clock), so this one spends as few as it can.
+//
+// Residual: the displacement gradient and its transpose go direction by
+// direction (24 instead of 243 FMAs per component and point), the reference
+// geometry is read back (152 bytes per point) instead of formed again, and all
+// warps of a CTA evaluate material points.  2898 elements with a time state:
+// 108 us; with a CTA per element, whose 27 material threads out of 256 also
+// formed the geometry, 1348 us.
+//
+// Tangent: dP/dF is pulled back to the reference coordinates, D_ijkl = w detJ0
+// sum_JL J0i_jJ A_iJkL J0i_lL, and summed against the products of the 1-D
+// tables direction by direction.  A lane owns (a_x, b_x, a_y) of one component
+// (i, k) and all (b_y, a_z, b_z).  Per point plane z and line y it forms the
+// nine sums over x, merges those that share their remaining factors into four
+// per b_y, and after the last line adds the plane to its 27 entries: 756 FMAs
+// per lane and component instead of 2187 per entry triple, and only the six
+// components i <= k (dP/dF is symmetric).  D lives in shared memory and is read
+// at one address per warp.  3456 elements: 1547 us against 7100 us by sums over all
+// 27 points and node pairs.  Five warps of 21 KB give ten per SM; that few
+// suffice because each FP64 warp instruction takes its SM partition 64 clocks.
+constexpr int H2_WARPS = 4, H2T_WARPS = 5;
+constexpr size_t H2T_SMEM = (size_t)H2T_WARPS * (27 * 81 + 2 * 9 * 27) * sizeof(double);
 
-__global__ void __launch_bounds__(32 * H2_WARPS)
-hex2_residual_kernel(MatParams mp, const int* __restrict__ elems, const double* __restrict__ geo,
-                     const double* __restrict__ d_full, const double* __restrict__ acc_full,
-                     double* __restrict__ rcontrib, int* __restrict__ status, int n_el) {
-  __shared__ double tab[2][9];                 // L, L' as [point][node]
-  __shared__ double buf[H2_WARPS][2][9 * 27];  // stage buffers
+template <bool TANGENT>
+__global__ void __launch_bounds__(32 * (TANGENT ? H2T_WARPS : H2_WARPS), TANGENT ? 2 : 1)
+hex2_element_kernel(MatParams mp, const int* __restrict__ elems, const double* __restrict__ geo,
+                    const double* __restrict__ d_full, const double* __restrict__ acc_full,
+                    double* __restrict__ rcontrib, double* __restrict__ contrib, int* __restrict__ status,
+                    int n_el) {
+  constexpr int WARPS = TANGENT ? H2T_WARPS : H2_WARPS;
+  __shared__ double tab[2][9];  // L, L' as [point][node]
+  // stage buffers, and (tangent) [point][81] of dP/dF
+  __shared__ double buf_static[TANGENT ? 1 : WARPS * 2 * 9 * 27];
+  extern __shared__ double hex2_smem[];
+  double* const bufs = TANGENT ? hex2_smem + WARPS * 27 * 81 : buf_static;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x < 9) {
     tab[0][threadIdx.x] = c_L[1][threadIdx.x / 3][threadIdx.x % 3];
     tab[1][threadIdx.x] = c_dL[1][threadIdx.x / 3][threadIdx.x % 3];
   }
   __syncthreads();
-  const int64_t e = blockIdx.x * (int64_t)H2_WARPS + warp;
+  const int64_t e = blockIdx.x * (int64_t)WARPS + warp;
   if (e >= n_el) return;
   const bool on = lane < 27;
   const int l = on ? lane : 0;
   const int x = l % 3, y = (l / 3) % 3, z = l / 9;
-  double (*b0)[27] = reinterpret_cast<double (*)[27]>(buf[warp][0]);
-  double (*b1)[27] = reinterpret_cast<double (*)[27]>(buf[warp][1]);
+  double (*b0)[27] = reinterpret_cast<double (*)[27]>(bufs + warp * 2 * 9 * 27);
+  double (*b1)[27] = reinterpret_cast<double (*)[27]>(bufs + (warp * 2 + 1) * 9 * 27);
+  double* const A = TANGENT ? hex2_smem + (warp * 27 + l) * 81 : nullptr;
   const double* L = tab[0];
   const double* D = tab[1];
   const int64_t node = elems[e * 27 + l];
@@ -636,8 +508,32 @@ hex2_residual_kernel(MatParams mp, const int* __restrict__ elems, const double* 
       for (int J = 0; J < 3; ++J)
         F[i][J] = (i == J ? 1.0 : 0.0) + H[0] * J0i[0][J] + H[1] * J0i[1][J] + H[2] * J0i[2][J];
     }
-    const bool ok = wd > 0.0 && material_point(mp, F, R, P, nullptr);
+    const bool ok = on && wd > 0.0 && material_point(mp, F, R, P, A);
     if (on && !ok) atomicOr(status, DEV_INVERTED);
+    if (TANGENT && on) {
+      // D in place of A: entry (3 i + j) 9 + 3 k + l, i <= k
+#pragma unroll 1
+      for (int ik = 0; ik < 9; ++ik) {
+        const int i = ik / 3, k = ik % 3;
+        if (i > k) continue;
+        double* a = A + 27 * i + 3 * k;
+        double B[3][3], C[3][3];
+#pragma unroll
+        for (int J = 0; J < 3; ++J)
+#pragma unroll
+          for (int M = 0; M < 3; ++M) B[J][M] = ok ? a[9 * J + M] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+          for (int M = 0; M < 3; ++M)
+            C[j][M] = wd * (J0i[j][0] * B[0][M] + J0i[j][1] * B[1][M] + J0i[j][2] * B[2][M]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+          for (int m = 0; m < 3; ++m)
+            a[9 * j + m] = C[j][0] * J0i[m][0] + C[j][1] * J0i[m][1] + C[j][2] * J0i[m][2];
+      }
+    }
     // Q_ij = w detJ0 sum_J P_iJ J0i_jJ, reusing F
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -712,6 +608,84 @@ hex2_residual_kernel(MatParams mp, const int* __restrict__ elems, const double* 
   }
   if (on)
     for (int i = 0; i < 3; ++i) rcontrib[(e * 27 + l) * 3 + i] = r[i];
+  if constexpr (TANGENT) {
+    __syncwarp();
+    if (on) b0[0][l] = mp.rho_dt2 * wd;  // consistent mass, on the diagonal i = k
+    __syncwarp();
+    if (!on) return;
+    const int ax = x, bx = y, ay = z;
+    double tnn[3], tnd[3], tdn[3], tdd[3];  // factors of a_x and b_x (d: derivative)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      tnn[q] = L[3 * q + ax] * L[3 * q + bx];
+      tnd[q] = L[3 * q + ax] * D[3 * q + bx];
+      tdn[q] = D[3 * q + ax] * L[3 * q + bx];
+      tdd[q] = D[3 * q + ax] * D[3 * q + bx];
+    }
+    const double* Dw = hex2_smem + warp * 27 * 81;
+    double* out = contrib + e * (27 * 27 * 9);
+#pragma unroll 1
+    for (int ik = 0; ik < 9; ++ik) {
+      const int i = ik / 3, k = ik % 3;
+      if (i > k) continue;
+      double K[3][3][3];  // b_y, a_z, b_z
+#pragma unroll
+      for (int t = 0; t < 27; ++t) K[t / 9][(t / 3) % 3][t % 3] = 0.0;
+#pragma unroll 1
+      for (int qz = 0; qz < 3; ++qz) {
+        double u[2][2][3];  // a_z derived, b_z derived, b_y
+#pragma unroll
+        for (int t = 0; t < 12; ++t) u[t / 6][(t / 3) % 2][t % 3] = 0.0;
+#pragma unroll 1
+        for (int qy = 0; qy < 3; ++qy) {
+          const int p = 3 * (qy + 3 * qz);
+          const double* d = Dw + p * 81 + 27 * i + 3 * k;
+          double s[3][3];  // sums over x of component (j, l)
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+              const double* t = j == 0 ? (m == 0 ? tdd : tdn) : (m == 0 ? tnd : tnn);
+              s[j][m] = t[0] * d[9 * j + m] + t[1] * d[81 + 9 * j + m] + t[2] * d[162 + 9 * j + m];
+            }
+          const double la = L[3 * qy + ay], da = D[3 * qy + ay];
+          double c0[3], c1[3];
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            c0[m] = la * s[0][m] + da * s[1][m];
+            c1[m] = la * s[2][m];
+          }
+          if (inertia && i == k)
+            c0[0] += la * (tnn[0] * b0[0][p] + tnn[1] * b0[0][p + 1] + tnn[2] * b0[0][p + 2]);
+#pragma unroll
+          for (int by = 0; by < 3; ++by) {
+            const double lb = L[3 * qy + by], db = D[3 * qy + by];
+            u[0][0][by] += lb * c0[0] + db * c0[1];
+            u[0][1][by] += lb * c0[2];
+            u[1][0][by] += lb * c1[0] + db * c1[1];
+            u[1][1][by] += lb * c1[2];
+          }
+        }
+#pragma unroll
+        for (int az = 0; az < 3; ++az) {
+          const double la = L[3 * qz + az], da = D[3 * qz + az];
+#pragma unroll
+          for (int by = 0; by < 3; ++by) {
+            const double d0 = la * u[0][0][by] + da * u[1][0][by], d1 = la * u[0][1][by] + da * u[1][1][by];
+#pragma unroll
+            for (int bz = 0; bz < 3; ++bz) K[by][az][bz] += L[3 * qz + bz] * d0 + D[3 * qz + bz] * d1;
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 27; ++t) {
+        const int by = t / 9, az = (t / 3) % 3, bz = t % 3;
+        const int a = ax + 3 * (ay + 3 * az), b = bx + 3 * (by + 3 * bz);
+        out[(a * 27 + b) * 9 + 3 * i + k] = K[by][az][bz];
+        if (i != k) out[(b * 27 + a) * 9 + 3 * k + i] = K[by][az][bz];
+      }
+    }
+  }
 }
 
 // Quadrature-point-parallel element kernel for elements with few points
@@ -1171,11 +1145,17 @@ void assemble(fem_problem* P, const double* d, double lam, double* residual, boo
                                                               accf, P->rcontrib.p, P->contrib.p, P->status.p, wt,
                                                               P->n_el);
   } else if (!want_tangent) {
-    hex2_residual_kernel<<<cdiv(P->n_el, H2_WARPS), 32 * H2_WARPS, 0, s>>>(
-        mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, P->status.p, P->n_el);
+    hex2_element_kernel<false><<<cdiv(P->n_el, H2_WARPS), 32 * H2_WARPS, 0, s>>>(
+        mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, nullptr, P->status.p, P->n_el);
   } else {
-    element_kernel<2, 256><<<P->n_el, 256, 0, s>>>(mp, P->coords.p, P->elems.p, fib, P->d_full.p,
-                                                    accf, P->rcontrib.p, P->contrib.p, P->status.p, wt);
+    static bool attr = false;
+    if (!attr) {
+      CB_CUDA(cudaFuncSetAttribute(hex2_element_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)H2T_SMEM));
+      attr = true;
+    }
+    hex2_element_kernel<true><<<cdiv(P->n_el, H2T_WARPS), 32 * H2T_WARPS, H2T_SMEM, s>>>(
+        mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, P->contrib.p, P->status.p, P->n_el);
   }
   CB_LAUNCH();
   {
