@@ -341,10 +341,11 @@ typedef struct {
 
 /* Flexible GMRES (right preconditioned by BDDC) for K x = b with the last
    assembled tangent of P.  Arnoldi step in FP64: for n_free <= 10^6 and
-   at most 128 basis vectors classical Gram-Schmidt applied twice, else
+   at most 256 basis vectors classical Gram-Schmidt applied twice, else
    modified Gram-Schmidt.  b, x:
-   dev [n_free]; x is overwritten (zero initial guess).  Synchronises once
-   per iteration to test convergence.  Returns CBDDC_ENOCONV if max_iters
+   dev [n_free]; x is overwritten (zero initial guess).  Reads the residual
+   back once per iteration to test convergence, with at most one further
+   iteration launched by then.  Returns CBDDC_ENOCONV if max_iters
    is reached. */
 CBDDC_API int gmres_solve(fem_problem* P, bddc_ctx* C, const double* b, double* x,
                 const gmres_options* opt, gmres_report* rep,

@@ -30,6 +30,7 @@ constexpr int64_t kCoopMaxN = 1000000;  // longest vector for the cooperative or
 // 388 and 341 us at 608k.
 constexpr int64_t kChunkMaxN = 300000;
 constexpr int MAXV = 128;       // Krylov vectors of the cooperative orthogonalisation
+constexpr int MAXT = 256;       // Krylov vectors of its tiled form
 constexpr int MAXR = 1024;      // Krylov vectors per cycle (restart <= MAXR - 1)
 
 __device__ inline double wsum(double v) {
@@ -360,7 +361,7 @@ __device__ void cgs_update(const CgsArgs& a, double* __restrict__ ws, double* __
 // sums of every CTA's partials into out[0:nout] (shared memory): every warp
 // 32 columns over every WARPS-th CTA, combined in a fixed order (identical
 // on every CTA, independent of scheduling)
-template <int WARPS>
+template <int WARPS, int NV>
 __device__ void cgs_reduce(const double* part, int nout, double* psum, double* out) {
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   for (int j0 = 0; j0 < nout; j0 += 32) {
@@ -368,7 +369,7 @@ __device__ void cgs_reduce(const double* part, int nout, double* psum, double* o
     double s = 0.0;
     if (j < nout) {
 #pragma unroll 4
-      for (unsigned c = grp; c < gridDim.x; c += WARPS) s += __ldcg(part + (int64_t)c * MAXV + j);
+      for (unsigned c = grp; c < gridDim.x; c += WARPS) s += __ldcg(part + (int64_t)c * NV + j);
     }
     psum[grp * 33 + lane] = s;
     __syncthreads();
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
     d.finish(a, psum, part);
   }
   grid.sync();
-  cgs_reduce<CGS_WARPS>(a.part, a.nvec, psum, h1);
+  cgs_reduce<CGS_WARPS, MAXV>(a.part, a.nvec, psum, h1);
   {
     CgsDots d(a.nvec);
     const int tile = a.js > 1 ? rows : CGS_TILE;
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
     d.finish(a, psum, part + stride);
   }
   grid.sync();
-  cgs_reduce<CGS_WARPS>(a.part + stride, a.nvec, psum, h2);
+  cgs_reduce<CGS_WARPS, MAXV>(a.part + stride, a.nvec, psum, h2);
   cgs_update(a, ws, upd, r0, 0, rows, h2);
   {
     double s = 0.0;
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
     }
   }
   grid.sync();
-  cgs_reduce<CGS_WARPS>(a.part + 2 * stride, 1, psum, wn2s);
+  cgs_reduce<CGS_WARPS, MAXV>(a.part + 2 * stride, 1, psum, wn2s);
   if (blockIdx.x == 0)
     givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, h1, h2, wn2s[0], a.scal, a.rtol, a.done, a.iters, psum);
   // v_{j+1} = w / ||w|| (the same value on every CTA)
@@ -438,13 +439,17 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
 }
 
 // The same step for vectors above kChunkMaxN unknowns, where V streams from
-// HBM: 256-row tiles dealt round-robin, w in global memory, a row per thread in
+// HBM, and for bases of MAXV to MAXT vectors: 256-row tiles dealt round-robin, w in global memory, a row per thread in
 // the updates and whole columns per warp in the dots.  Neighbouring CTAs then
 // read neighbouring tiles of the same column, which HBM serves better than the
-// chunks' 304 distant streams, and the FMAs hide behind it.
+// chunks' 304 distant streams, and the FMAs hide behind it.  Past MAXV vectors
+// it replaces modified Gram-Schmidt, whose grid-wide barrier per vector cost
+// more than the second pass: 924 us against 1100 us at n = 582k and 147 vectors,
+// 397 us against 1404 us at n = 27k and 192 vectors.
+template <int NV>
 __device__ void tiles_phase(const CgsArgs& a, const double* hin, bool norm, double* ws, double* part) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int CPW = MAXV / (DOT_THREADS / 32);  // columns per warp
+  constexpr int CPW = NV / (DOT_THREADS / 32);  // columns per warp
   double acc[CPW];
 #pragma unroll
   for (int q = 0; q < CPW; ++q) acc[q] = 0.0;
@@ -482,33 +487,35 @@ __device__ void tiles_phase(const CgsArgs& a, const double* hin, bool norm, doub
     if (tid == 0) {
       double sm = 0.0;
       for (int q = 0; q < DOT_THREADS / 32; ++q) sm += red[q];
-      part[(int64_t)blockIdx.x * MAXV] = sm;
+      part[(int64_t)blockIdx.x * NV] = sm;
     }
   } else {
 #pragma unroll
     for (int q = 0; q < CPW; ++q) {
       const int j = warp + (DOT_THREADS / 32) * q;
       const double v = wsum(acc[q]);
-      if (lane == 0 && j < a.nvec) part[(int64_t)blockIdx.x * MAXV + j] = v;
+      if (lane == 0 && j < a.nvec) part[(int64_t)blockIdx.x * NV + j] = v;
     }
   }
 }
 
-__global__ void __launch_bounds__(DOT_THREADS) cgs2_tiles_kernel(CgsArgs a) {
+template <int NV>
+__global__ void __launch_bounds__(DOT_THREADS, 2) cgs2_tiles_kernel(CgsArgs a) {
   cg::grid_group grid = cg::this_grid();
   if (*a.done) return;  // read by every CTA before any barrier: uniform
-  __shared__ double ws[DOT_THREADS], psum[DOT_THREADS / 32 * 33 > 3 * MAXV ? DOT_THREADS / 32 * 33 : 3 * MAXV];
-  __shared__ double h1[MAXV], h2[MAXV], wn2s[1];
-  const int64_t stride = (int64_t)gridDim.x * MAXV;
-  tiles_phase(a, nullptr, false, ws, a.part);
+  __shared__ double ws[DOT_THREADS], psum[3 * NV];
+  static_assert(3 * NV >= DOT_THREADS / 32 * 33, "reduction scratch");
+  __shared__ double h1[NV], h2[NV], wn2s[1];
+  const int64_t stride = (int64_t)gridDim.x * NV;
+  tiles_phase<NV>(a, nullptr, false, ws, a.part);
   grid.sync();
-  cgs_reduce<DOT_THREADS / 32>(a.part, a.nvec, psum, h1);
-  tiles_phase(a, h1, false, ws, a.part + stride);
+  cgs_reduce<DOT_THREADS / 32, NV>(a.part, a.nvec, psum, h1);
+  tiles_phase<NV>(a, h1, false, ws, a.part + stride);
   grid.sync();
-  cgs_reduce<DOT_THREADS / 32>(a.part + stride, a.nvec, psum, h2);
-  tiles_phase(a, h2, true, ws, a.part + 2 * stride);
+  cgs_reduce<DOT_THREADS / 32, NV>(a.part + stride, a.nvec, psum, h2);
+  tiles_phase<NV>(a, h2, true, ws, a.part + 2 * stride);
   grid.sync();
-  cgs_reduce<DOT_THREADS / 32>(a.part + 2 * stride, 1, psum, wn2s);
+  cgs_reduce<DOT_THREADS / 32, NV>(a.part + 2 * stride, 1, psum, wn2s);
   if (blockIdx.x == 0)
     givens_update(a.j, a.m, a.H, a.cs, a.sn, a.g, h1, h2, wn2s[0], a.scal, a.rtol, a.done, a.iters, psum);
   // v_{j+1} = w / ||w|| (the same value on every CTA)
@@ -721,8 +728,7 @@ void Gmres::ensure(int64_t n_, int m_) {
     CB_CUDA(cudaGetDevice(&dev));
     CB_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     CB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    coop_grid = 0;
-    cgs_rows = 0;
+    coop_grid = tile_grid = 0;
     if (coop && n_ <= kChunkMaxN) {
       // two CTAs per SM, fewer for short vectors: the FMAs shrink with the
       // grid and the sums of its partials grow with it
@@ -733,14 +739,16 @@ void Gmres::ensure(int64_t n_, int m_) {
       cgs_js = (int)std::min<int64_t>(CGS_JS, std::max<int64_t>(1, 4 * CGS_WARPS / (cgs_rows / 32)));
       cgs_smem = (size_t)cgs_rows * (cgs_js > 1 ? 1 + cgs_js : 1) * sizeof(double);
       CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_coop_kernel, CGS_THREADS, cgs_smem));
-      if (coop_grid > per_sm * sms) coop_grid = cgs_rows = 0;
+      if (coop_grid > per_sm * sms) coop_grid = 0;
     }
-    if (coop && n_ <= kCoopMaxN && coop_grid == 0) {
-      CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_tiles_kernel, DOT_THREADS, 0));
-      coop_grid = (int)std::min<int64_t>(std::min(per_sm, 2) * (int64_t)sms,
+    if (coop && n_ <= kCoopMaxN) {
+      // at most two CTAs per SM, about four row tiles per CTA
+      CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_tiles_kernel<MAXT>, DOT_THREADS, 0));
+      tile_grid = (int)std::min<int64_t>(std::min(per_sm, 2) * (int64_t)sms,
                                          std::max<int64_t>(1, cdiv(n_, DOT_THREADS) / 4));
     }
-    if (coop_grid > 0) cpart.alloc((size_t)3 * coop_grid * MAXV);
+    if (coop_grid + tile_grid > 0)
+      cpart.alloc(3 * std::max((size_t)coop_grid * MAXV, (size_t)tile_grid * MAXT));
     // MGS cooperative launch: one CTA of MGS_THREADS per SM, rows per
     // thread rounded up to 8, 16, 24 or 32 (n up to 3.1M on 152 SMs; 0:
     // the multi-launch path)
@@ -844,15 +852,17 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
     double* h2 = G.h.p + G.hstride;
     double* wn2 = G.h.p + 2 * G.hstride;
     timer_begin(CBDDC_TIMER_ORTH, s);
-    if (G.coop_grid > 0 && j + 1 <= MAXV) {
-      // short vectors and bases: CGS2 in one cooperative launch
+    const bool chunks = G.coop_grid > 0 && j + 1 <= MAXV;
+    if (chunks || (G.tile_grid > 0 && j + 1 <= MAXT)) {
+      // CGS2 in one cooperative launch
       CgsArgs ca{G.V.p, n, j + 1, G.cgs_rows, G.cgs_js, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.cpart.p, j, m,
                  G.H.p, G.cs.p, G.sn.p, G.g.p, G.scal.p, rtol, done, kcount};
       void* args[] = {&ca};
-      const bool chunks = G.cgs_rows > 0;
-      CB_CUDA(cudaLaunchCooperativeKernel(chunks ? (const void*)cgs2_coop_kernel : (const void*)cgs2_tiles_kernel,
-                                          dim3(G.coop_grid), dim3(chunks ? CGS_THREADS : DOT_THREADS), args,
-                                          chunks ? G.cgs_smem : 0, s));
+      const void* fn = chunks          ? (const void*)cgs2_coop_kernel
+                       : j + 1 <= MAXV ? (const void*)cgs2_tiles_kernel<MAXV>
+                                       : (const void*)cgs2_tiles_kernel<MAXT>;
+      CB_CUDA(cudaLaunchCooperativeKernel(fn, dim3(chunks ? G.coop_grid : G.tile_grid),
+                                          dim3(chunks ? CGS_THREADS : DOT_THREADS), args, chunks ? G.cgs_smem : 0, s));
       CB_LAUNCH();
     } else if (G.mgs_grid > 0) {
       MgsArgs ma{G.V.p, n, G.w.p, G.V.p + (int64_t)(j + 1) * n, G.mpart.p, G.h.p, j, m,
@@ -913,8 +923,8 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
     if (total >= max_iters) break;
     // The host reads the residual of every step.  Waiting for it before the
     // next step is launched left the GPU idle for the copy, the wake-up and the
-    // first launches (25-55 us of each 200-350 us step on the smaller meshes),
-    // so one further step is launched before step j's residual is known,
+    // first launches (4 to 6 us of each 170 to 440 us step of 27k unknowns), so
+    // one further step is launched before step j's residual is known,
     // unless that residual can be expected to end the solve (one step gains
     // less than a factor of five): a step launched too many is skipped by the
     // Gram-Schmidt kernels, at the price of its apply and product.

@@ -19,8 +19,9 @@ struct Gmres {
   int* flags() const { return reinterpret_cast<int*>(scal.p + 8); }
   DVec<unsigned> ticket;
   DVec<double> cpart;        // per-CTA partials of the cooperative orthogonalisation
-  int coop_grid = 0;         // its grid size (0: use the multi-launch path)
-  int cgs_rows = 0, cgs_js = 1;  // rows per CTA and column parts of the update (0: tiles)
+  int coop_grid = 0;         // its grid with a chunk of w per CTA (0: not available)
+  int cgs_rows = 0, cgs_js = 1;  // rows per CTA and column parts of the update
+  int tile_grid = 0;         // its grid over row tiles (0: not available)
   size_t cgs_smem = 0;
   DVec<double> mpart;        // per-CTA partials of the cooperative MGS step
   int mgs_grid = 0, mgs_rpt = 0;  // its grid and rows per thread (0: not available)

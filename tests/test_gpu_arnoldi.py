@@ -47,11 +47,11 @@ def test_gmres_against_dense_solve(n, restart):
     assert torch.equal(x, y)
 
 
-@pytest.mark.parametrize("n", [(5, 3, 3), (11, 8, 8)])
-def test_basis_past_the_classical_step(n):
-    # 200 vectors whatever the residual: the steps past 128 take the modified
-    # Gram-Schmidt kernel (here most of its CTAs own no row), and the least
-    # squares solution must stay the converged one
+@pytest.mark.parametrize("n,m", [((5, 3, 3), 200), ((11, 8, 8), 200), ((7, 7, 7), 257), ((11, 8, 8), 300)])
+def test_basis_past_the_chunked_step(n, m):
+    # m vectors whatever the residual: the steps past 128 take the tiled
+    # kernel, those past 256 modified Gram-Schmidt (here most of its CTAs own no
+    # row), and the least squares solution must stay the converged one
     prob = slab_problem(*n, order=1, lengths=tuple(0.2 * k for k in n), parts=(2, 1, 1), jitter=0.1, primal="VEF")
     fe = FEProblem(prob)
     d = np.zeros(fe.n_free)
@@ -60,7 +60,7 @@ def test_basis_past_the_classical_step(n):
     pc = pkg.BDDC(P, precision=pkg.FP64, primal="VEF").setup()
     b = np.random.default_rng(11).standard_normal(fe.n_free)
     x = torch.empty(fe.n_free, dtype=torch.float64, device="cuda")
-    rep = pc.gmres(torch.as_tensor(b, device="cuda"), x, restart=200, max_iters=200, rtol=1e-300)
-    assert rep["iterations"] == 200 and not rep["converged"]
+    rep = pc.gmres(torch.as_tensor(b, device="cuda"), x, restart=m, max_iters=m, rtol=1e-300)
+    assert rep["iterations"] == m and not rep["converged"]
     ref = np.linalg.solve(fe.tangent(d, 0.6)[0].toarray(), b)
     assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-8 * np.linalg.norm(ref)
