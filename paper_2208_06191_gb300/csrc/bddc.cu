@@ -1776,6 +1776,33 @@ static void panel_launch(int n, int nmat, cudaStream_t s, const SweepDesc* desc,
   if (!wide) panel_launch_ch<T, NB, NP, 16>(n, nmat, s, desc, k, mat, Pbuf, X, Y, lo);
 }
 
+// Pivot block inverses of step k: FP64 blocks of few matrices over clusters
+// (measured at the kernel).
+template <typename T, int NB>
+static void diag_launch(int nmat, cudaStream_t s, const SweepDesc* desc, int k, T* mat, T* Pbuf, int* status,
+                        double tol) {
+  if constexpr (sizeof(T) == 8) {
+    if (DIAG_CLUSTER * nmat <= 152) {
+      constexpr int RW = 4;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(DIAG_CLUSTER * nmat);
+      cfg.blockDim = dim3(DiagThreads<NB, DIAG_CLUSTER, RW>::value);
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = DIAG_CLUSTER;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      CB_CUDA(cudaLaunchKernelEx(&cfg, sweep_diag_kernel<T, NB, DIAG_CLUSTER, RW>, desc, k, mat, Pbuf, status, tol));
+      CB_LAUNCH();
+      return;
+    }
+  }
+  sweep_diag_kernel<T, NB, 1, 8><<<nmat, DiagThreads<NB, 1, 8>::value, 0, s>>>(desc, k, mat, Pbuf, status, tol);
+  CB_LAUNCH();
+}
+
 // One sweep: per pivot block the diagonal inverse, the panels and the
 // rank-NB update.  FP32 lists bound to the tensor cores get their panels as
 // split TF32 operands (X, Xlo, Y^T, Ylo) and skip the split pass.
@@ -1787,8 +1814,7 @@ static void run_sweep_nb(const DVec<SweepDesc>& desc, int nmat, const std::vecto
                          cudaStream_t s, T* const* lo) {
   T* const none[4] = {nullptr, nullptr, nullptr, nullptr};
   for (int k = 0; k < (int)lists.size(); ++k) {
-    sweep_diag_kernel<T, NB><<<nmat, DiagThreads<NB>::value, 0, s>>>(desc.p, k, mat, Pbuf, status, tol);
-    CB_LAUNCH();
+    diag_launch<T, NB>(nmat, s, desc.p, k, mat, Pbuf, status, tol);
     const int n = std::max(maxRows, maxCols);
     const bool split = sizeof(T) == 4 && lists[k].presplit && lists[k].tc_bound && tensor_cores_for(true);
     bool formed = false;

@@ -9,14 +9,16 @@
 // Section 3.2 in one pass; sweeping a whole matrix inverts it.
 //
 // Pivot block k (rows/cols kk of width kb <= NB) is processed as
-//   P = A_kk^-1 (one CTA per matrix, FP64 Gauss-Jordan in shared memory),
+//   P = A_kk^-1 (a CTA or a cluster per matrix, Gauss-Jordan),
 //   X = A[:, kk] with X[kk] = -I,   Y = P A[kk, :] with Y[:, kk] = P,
 //   A[kk, :] = 0, A[:, kk] = 0,     A -= X Y   (grouped GEMM, K = kb),
 // which is the rank-kb form of the sweep.  No pivoting: a pivot below
 // tol * max|diag| (or non-finite) sets DEV_PIVOT in the status word.
 #pragma once
-#include <memory>
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <memory>
 #include <vector>
 
 #include "common.h"
@@ -648,21 +650,38 @@ struct SweepDesc {
 // least); 95 us measured, 166 us when every warp formed the reciprocal behind
 // the barrier.  FP32: bound by the chain (barrier, reciprocal, broadcast),
 // 22 us against 39 us.
-template <int NB>
-struct DiagThreads { static constexpr int value = 4 * NB; };
-template <typename T, int NB>
-__global__ void __launch_bounds__(DiagThreads<NB>::value)
+//
+// CL > 1: the rows of one block go over a cluster of CL CTAs, RW rows per warp,
+// and the owner of the next row writes it into every CTA's shared memory before
+// the cluster barrier that takes the place of the CTA's.  The arithmetic of
+// every entry is the same.  A single SM's FP64 pipe is then no longer the
+// bound, but the chain of update, reciprocal and barrier: 79 us for FP64 blocks
+// of 64 (one to a few matrices) against 95 us.  It pays while the matrices leave
+// SMs idle (DIAG_CLUSTER * matrices <= 152); with 64 and 512 matrices both forms
+// take the same time (99 and 94 us).
+constexpr int DIAG_CLUSTER = 4;
+template <int NB, int CL, int RW>
+struct DiagThreads { static constexpr int value = 32 * NB / (RW * CL); };
+template <typename T, int NB, int CL, int RW>
+__global__ void __launch_bounds__(DiagThreads<NB, CL, RW>::value)
 sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat, T* __restrict__ Pbuf,
                   int* __restrict__ status, double tol) {
-  constexpr int RW = 8, CW = NB / 32;  // rows per warp, columns per lane
+  static_assert(RW % 2 == 0 && NB % (RW * CL) == 0, "rows per warp and CTA");
+  constexpr int CW = NB / 32;  // columns per lane
+  constexpr int WARPS = NB / (RW * CL);
   __shared__ __align__(16) T colb[2][NB];
   __shared__ T rowb[2][NB];
-  const SweepDesc d = desc[blockIdx.x];
+  const SweepDesc d = desc[blockIdx.x / CL];
   const int k0 = k * NB;
   if (k0 >= d.p) return;
   const int kb = min(NB, d.p - k0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // warp of the block's NB / RW, and its first row
+  const int warp = (int)(blockIdx.x % CL) * WARPS + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int r0 = RW * warp;
+  auto sync = [] {
+    if constexpr (CL > 1) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+  };
   const T* A = mat + d.off + (int64_t)k0 * d.ld + k0;
   T a[RW][CW];
 #pragma unroll
@@ -688,7 +707,13 @@ sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat
 #pragma unroll
     for (int v = 0; v < CW; ++v) {
       const int c = lane + 32 * v;
-      rowb[b][c] = c == j ? inv : r[v] * inv;
+      const T x = c == j ? inv : r[v] * inv;
+      if constexpr (CL > 1) {
+#pragma unroll
+        for (int q = 0; q < CL; ++q) *cooperative_groups::this_cluster().map_shared_rank(&rowb[b][c], q) = x;
+      } else {
+        rowb[b][c] = x;
+      }
     }
     if (!(fabs((double)pv) > tol * scale) || !isfinite((double)pv)) bad = true;
   };
@@ -702,6 +727,7 @@ sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat
         }
     }
   };
+  if constexpr (CL > 1) sync();  // every CTA of the cluster runs before its shared memory is written
   if (warp == 0) publish_row(a[0], 0, 0);
   publish_col(0, 0);
   for (int j0 = 0; j0 < kb; j0 += RW) {
@@ -709,11 +735,10 @@ sweep_diag_kernel(const SweepDesc* __restrict__ desc, int k, T* __restrict__ mat
     for (int u = 0; u < RW; ++u) {
       const int j = j0 + u;
       if (j >= kb) break;
-      constexpr int un_of[RW] = {1, 2, 3, 4, 5, 6, 7, 0};
-      const int un = un_of[u];                      // row of j + 1 in its warp
+      const int un = (u + 1) % RW;                  // row of j + 1 in its warp
       const int b = u & 1;
       const bool last = j + 1 >= kb;
-      __syncthreads();
+      sync();
       T t[CW], col[RW];
       bool own[CW];                                 // this lane's column is j
 #pragma unroll
