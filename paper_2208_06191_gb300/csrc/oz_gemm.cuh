@@ -337,17 +337,17 @@ gemm_kernel(const int4* __restrict__ tiles, int ntiles, const Prob* __restrict__
     int b = 0, g = 0;  // K blocks and TMEM tiles of this CTA so far
     bool ok = true;
     const uint64_t da0 = tc::sw128_desc(tc::smem_u32(sA)), db0 = tc::sw128_desc(tc::smem_u32(sB));
-    for (int i = 0; i < ntl && ok && !*(volatile int*)abort_flag; ++i) {
+    for (int i = 0; i < ntl && ok && !tc::warp_aborted(abort_flag); ++i) {
       const int4 tl = tiles[blockIdx.x + i * gridDim.x];
       const int nk = (probs[tl.x].K + BK - 1) / BK;
       for (int c = 0; c < nk && ok; ++c, ++b) {
-        for (int q = S - 1; q >= 0 && ok; --q) ok = tc::mbar_wait(&full[q], b & 1);
+        for (int q = S - 1; q >= 0 && ok; --q) ok = tc::warp_wait(&full[q], b & 1);
         // orders from the highest down: slice k is free after order k
 #pragma unroll
         for (int k = S - 1; k >= 0; --k, ++g) {
           const int a = g % SLOTS;
           if (!ok) break;
-          if (g >= SLOTS && !tc::mbar_wait(&sempty[a], (g / SLOTS - 1) & 1)) {
+          if (g >= SLOTS && !tc::warp_wait(&sempty[a], (g / SLOTS - 1) & 1)) {
             ok = false;
             break;
           }
@@ -394,7 +394,7 @@ gemm_kernel(const int4* __restrict__ tiles, int ntiles, const Prob* __restrict__
 #pragma unroll
         for (int k = S - 1; k >= 0; --k, ++g) {
           const int a = g % SLOTS;
-          if (!tc::mbar_wait(&sfull[a], (g / SLOTS) & 1) || *(volatile int*)abort_flag) {
+          if (!tc::warp_wait(&sfull[a], (g / SLOTS) & 1) || tc::warp_aborted(abort_flag)) {
             ok = false;
             break;
           }

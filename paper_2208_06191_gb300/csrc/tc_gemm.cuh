@@ -97,9 +97,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 }
 
 // Bounded wait for the phase with the given parity; false on expiry.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = kWaitLimit) {
   const uint32_t a = smem_u32(bar);
-  for (uint32_t it = 0; it < kWaitLimit; ++it) {
+  for (uint32_t it = 0; it < limit; ++it) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -110,6 +110,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     if (ok) return true;
   }
   return false;
+}
+
+// The same for a whole converged warp, with one answer for all its lanes: true
+// if every lane saw the phase end.  The lanes poll on their own and can differ
+// near the limit; what follows a wait (elect.sync, tcgen05.ld, votes,
+// __syncwarp) needs all of them, so that a warp that split there would hang
+// where the limit is to end the kernel.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint32_t limit = kWaitLimit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
+}
+
+// Whether another warp gave up, with one answer for all lanes of a converged
+// warp (the flag can be set between the reads of two lanes).
+__device__ __forceinline__ bool warp_aborted(const int* flag) {
+  return __any_sync(0xffffffffu, *(const volatile int*)flag != 0);
 }
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
@@ -304,12 +319,12 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
     // lane every MMA cost about 100 clocks).
     int g = 0;  // TMEM slices of this CTA so far (SPC per operand chunk)
     bool ok = true;
-    for (int i = 0; i < ntl && ok && !*(volatile int*)abort_flag; ++i) {
+    for (int i = 0; i < ntl && ok && !warp_aborted(abort_flag); ++i) {
       const int4 tl = tiles[blockIdx.x + i * gridDim.x];
       const int nk = (probs[tl.x].K + BKC - 1) / BKC;
       for (int c = 0; c < nk && ok; ++c) {
         const int s = (g / SPC) % NST;  // operand stage of chunk c (g counts slices)
-        if (!mbar_wait(&full[s], ((g / SPC) / NST) & 1)) {
+        if (!warp_wait(&full[s], ((g / SPC) / NST) & 1)) {
           ok = false;
           break;
         }
@@ -319,7 +334,7 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
         for (int sl = 0; sl < SPC; ++sl, ++g) {
           const int a = g & 1;
           if (!ok) break;
-          if (g >= 2 && !mbar_wait(&sempty[a], ((g >> 1) - 1) & 1)) {
+          if (g >= 2 && !warp_wait(&sempty[a], ((g >> 1) - 1) & 1)) {
             ok = false;
             break;
           }
@@ -394,7 +409,7 @@ tc_gemm_kernel(const int4* __restrict__ tiles, int ntiles, const TcProb* __restr
       for (int q = 0; q < 64; ++q) rs[q] = 0.f;
       for (int c = 0; c < nk * SPC; ++c, ++g) {
         const int a = g & 1;
-        if (!mbar_wait(&sfull[a], (g >> 1) & 1) || *(volatile int*)abort_flag) {
+        if (!warp_wait(&sfull[a], (g >> 1) & 1) || warp_aborted(abort_flag)) {
           ok = false;
           break;
         }
