@@ -1334,14 +1334,25 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
   // The constraint matrix G = C S_rr^-1 C^T (n_a x n_a) is inverted by a
   // third sweep; its panels fit the same X / Y buffers (n_a <= n_s rows,
   // ld_G <= ld_A columns).
-  std::vector<SweepDesc> sw1(nsub), sw2(nsub), swg(nsub);
+  std::vector<SweepDesc> sw1(nsub), sw2(nsub), swg(nsub), sgg(nsub);
+  // FP64 products: exponents along K (diag_exp_kernel) of A_II, of S, of the
+  // augmented S, of G and of the coarse or deluxe matrices, one after another.
+  // Symmetric scalings: op(A)(:, k) of size d_k (A_GI, Y, S, X panels) is
+  // divided by 2^kexp, of size 1 / d_k (inverses) multiplied, and Psi^T S Phi is
+  // scaled as (Psi^T d) (d^-1 S Phi).
+  const int64_t keI = 0, keS = C->totI, keW = keS + C->totG, keA = keW + C->totG;
+  int64_t nke = keA + C->totC;
   for (int s = 0; s < nsub; ++s) {
     sw1[s] = SweepDesc{C->nI[s], C->nI[s], C->ldA[s], C->nI[s], C->offA[s], C->offX[s], C->offYp[s],
-                       C->offP[s]};
+                       C->offP[s], keI + C->offI[s]};
     sw2[s] = SweepDesc{C->nG[s], C->nG[s], C->ldS[s], C->nr[s], C->offS[s], C->offX[s], C->offYp[s],
-                       C->offP[s]};
+                       C->offP[s], keW + C->offGam[s]};
     swg[s] = SweepDesc{C->na[s], C->na[s], C->ldG[s], C->na[s], C->offG[s], C->offX[s], C->offYp[s],
-                       C->offP[s]};
+                       C->offP[s], keA + C->offC[s]};
+    // (the block A_GG, which holds S after the interior elimination; not swept)
+    sgg[s] = SweepDesc{C->nG[s], C->nG[s], C->ldA[s], 0,
+                       C->offA[s] + (int64_t)C->nI[s] * C->ldA[s] + round_up(C->nI[s], 4), 0, 0, 0,
+                       keS + C->offGam[s]};
     C->steps1 = std::max(C->steps1, (int)cdiv(C->nI[s], NB));
     C->steps2 = std::max(C->steps2, (int)cdiv(C->nr[s], NB));
     C->stepsg = std::max(C->stepsg, (int)cdiv(C->na[s], NB));
@@ -1349,6 +1360,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
   C->sw1.upload(sw1);
   C->sw2.upload(sw2);
   C->swg.upload(swg);
+  if (C->esize == 8) C->sgg.upload(sgg);
   const int to_sw = C->tile_order;
   auto sweep_gemms = [NB, es, to_sw](const std::vector<SweepDesc>& sw, int steps, std::vector<GemmList>& out) {
     const int to = to_sw;
@@ -1361,8 +1373,9 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       for (int s = 0; s < nmat; ++s) {
         const SweepDesc& d = sw[s];
         const int kb = std::max(0, std::min(NB, d.p - k * NB));
-        g.push_back(GemmProb{d.rows, d.cols, kb, NB, d.ld, d.ld, d.offX, d.offY, d.off});
-        y.push_back(GemmProb{kb, d.cols, kb, NB, d.ld, d.ld, d.offP, d.off + (int64_t)k * NB * d.ld, d.offY});
+        const int64_t ke = d.ke + (int64_t)k * NB;
+        g.push_back(GemmProb{d.rows, d.cols, kb, NB, d.ld, d.ld, d.offX, d.offY, d.off, -1, ke});
+        y.push_back(GemmProb{kb, d.cols, kb, NB, d.ld, d.ld, d.offP, d.off + (int64_t)k * NB * d.ld, d.offY, 1, ke});
         if (kb > 0) cols += d.cols;
       }
       out[k].set(g, es, false, to);
@@ -1416,7 +1429,8 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       }
       dlx_flops += 2.0 * n * (double)n * n;
       coff[k + 1] = coff[k] + round_up((int64_t)n * ld, kAlign);
-      swd[k] = SweepDesc{n, n, ld, n, coff[k], xo, yo, (int64_t)k * NB * NB};
+      swd[k] = SweepDesc{n, n, ld, n, coff[k], xo, yo, (int64_t)k * NB * NB, nke};
+      nke += n;
       xo += round_up((int64_t)n * NB, kAlign);
       yo += round_up((int64_t)NB * ld, kAlign);
       C->stepsd = std::max(C->stepsd, (int)cdiv(n, NB));
@@ -1431,7 +1445,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
     std::vector<GemmProb> gd(nb);
     for (int k = 0; k < nk; ++k)
       for (int q = cptr[k]; q < cptr[k + 1]; ++q)
-        gd[q] = GemmProb{bn[q], bn[q], bn[q], bld[q], bld[q], bld[q], coff[k], boff[q], boff[q]};
+        gd[q] = GemmProb{bn[q], bn[q], bn[q], bld[q], bld[q], bld[q], coff[k], boff[q], boff[q], 1, swd[k].ke};
     C->gl_dlx.set(gd, es, false, C->tile_order);
     auto sz = [&](int64_t n) { return (size_t)(std::max<int64_t>(n, 1) + kAlign) * es; };
     C->Dsb.alloc(sz(boff[nb]));
@@ -1449,19 +1463,19 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
     const int64_t aII = C->offA[s], aIG = C->offA[s] + cI;
     const int64_t aGI = C->offA[s] + (int64_t)C->nI[s] * C->ldA[s], aGG = aGI + cI;
     gE.push_back(GemmProb{C->nI[s], C->nG[s], C->nI[s], C->ldA[s], C->ldA[s], C->ldS[s], aII, aIG,
-                          C->offE[s]});
+                          C->offE[s], 1, sw1[s].ke});
     gS.push_back(GemmProb{C->nG[s], C->nG[s], C->nI[s], C->ldA[s], C->ldS[s], C->ldA[s], aGI, C->offE[s],
-                          aGG});
+                          aGG, -1, sw1[s].ke});
     gW.push_back(GemmProb{C->na[s], C->nG[s], C->na[s], C->ldG[s], C->ldS[s], C->ldS[s], C->offG[s],
-                          C->offZ[s], C->offZ[s]});
+                          C->offZ[s], C->offZ[s], 1, swg[s].ke});
     gT.push_back(GemmProb{C->nr[s], C->nG[s], C->na[s], C->ldY[s], C->ldS[s], C->ldS[s], C->offY[s],
-                          C->offZ[s], C->offS[s]});
+                          C->offZ[s], C->offS[s], -1, swg[s].ke});
     gPA.push_back(GemmProb{C->nr[s], C->na[s], C->na[s], C->ldY[s], C->ldG[s], C->ldPhi[s], C->offY[s],
-                           C->offG[s], C->offPhi[s] + C->nv[s]});
+                           C->offG[s], C->offPhi[s] + C->nv[s], -1, swg[s].ke});
     gSP.push_back(GemmProb{C->nG[s], C->nc[s], C->nG[s], C->ldA[s], C->ldPhi[s], C->ldPhi[s], aGG,
-                           C->offPhi[s], C->offPhi[s]});
+                           C->offPhi[s], C->offPhi[s], -1, sgg[s].ke});
     gKc.push_back(GemmProb{C->nc[s], C->nc[s], C->nG[s], C->ldPhi[s], C->ldPhi[s], C->ldPhi[s],
-                           C->offPhi[s], C->offPhi[s], C->offKc[s]});
+                           C->offPhi[s], C->offPhi[s], C->offKc[s], 1, sgg[s].ke});
   }
   const int to = C->tile_order;
   C->gl_E.set(gE, es, false, to);
@@ -1479,7 +1493,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       const int cI = (int)round_up(C->nI[s], 4);
       const int64_t aGG = C->offA[s] + (int64_t)C->nI[s] * C->ldA[s] + cI;
       gPV.push_back(GemmProb{C->nr[s], C->nv[s], C->nr[s], C->ldS[s], C->ldA[s], C->ldPhi[s], C->offS[s],
-                             aGG + (int64_t)C->nr[s] * C->ldA[s], C->offPhi[s]});
+                             aGG + (int64_t)C->nr[s] * C->ldA[s], C->offPhi[s], 1, sgg[s].ke});
     }
     C->gl_PsiV.set(gPV, es, true, C->tile_order);
     C->Psi.alloc(sized(C->offPhi[nsub]));
@@ -1514,7 +1528,8 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
     C->ScX.alloc((size_t)C->n_pi * NBc);
     C->ScY.alloc((size_t)C->n_pi * NBc);
     C->ScP.alloc((size_t)NBc * NBc);
-    std::vector<SweepDesc> swc{SweepDesc{C->n_pi, C->n_pi, C->n_pi, C->n_pi, 0, 0, 0, 0}};
+    std::vector<SweepDesc> swc{SweepDesc{C->n_pi, C->n_pi, C->n_pi, C->n_pi, 0, 0, 0, 0, nke}};
+    nke += C->n_pi;
     C->swc.upload(swc);
     C->stepsc = (int)cdiv(C->n_pi, NBc);
     {
@@ -1525,7 +1540,8 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       for (int k = 0; k < C->stepsc; ++k) {
         const SweepDesc& d = swc[0];
         const int kb = std::max(0, std::min(NBc, d.p - k * NBc));
-        std::vector<GemmProb> g{GemmProb{d.rows, d.cols, kb, NBc, d.ld, d.ld, d.offX, d.offY, d.off}};
+        std::vector<GemmProb> g{GemmProb{d.rows, d.cols, kb, NBc, d.ld, d.ld, d.offX, d.offY, d.off, -1,
+                                         d.ke + (int64_t)k * NBc}};
         C->gl_swc[k].set(g, 8);
         (void)nmat;
       }
@@ -1694,7 +1710,8 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
     for (auto* g : lists) need = std::max(need, g->oz_bytes());
     if (need > 0) {
       C->oz_scratch.alloc((size_t)need);
-      for (auto* g : lists) g->bind_oz(C->oz_scratch.p, P->status.p);
+      C->kexp.alloc((size_t)nke);
+      for (auto* g : lists) g->bind_oz(C->oz_scratch.p, P->status.p, C->kexp.p);
     }
   }
   // FP32 contexts: one scratch buffer for the split operands of the
@@ -1836,13 +1853,26 @@ static void run_sweep_nb(const DVec<SweepDesc>& desc, int nmat, const std::vecto
   }
 }
 
+// Exponents along K of the FP64 products over the listed matrices, from their
+// diagonals.
+static void run_diag_exp(const DVec<SweepDesc>& desc, int nmat, int maxRows, const double* mat, int* kexp,
+                         cudaStream_t s) {
+  if (nmat == 0 || maxRows == 0) return;
+  diag_exp_kernel<<<dim3(cdiv(maxRows, 256), nmat), 256, 0, s>>>(desc.p, mat, kexp);
+  CB_LAUNCH();
+}
+
 // Sweep with pivot blocks of nb (64, or 128 for FP32 operators).
+// kexp: the context's exponents along K (FP64 with integer slices).
 template <typename T>
 static void run_sweep(const DVec<SweepDesc>& desc, int nmat, const std::vector<GemmList>& lists,
                       int maxRows, int maxCols, T* mat, T* X, T* Y, T* Pbuf, int* status, double tol,
-                      cudaStream_t s, int nb = SWEEP_NB, T* const* lo = nullptr) {
+                      cudaStream_t s, int* kexp, int nb = SWEEP_NB, T* const* lo = nullptr) {
   T* const none[4] = {nullptr, nullptr, nullptr, nullptr};
   if (!lo) lo = none;
+  if constexpr (sizeof(T) == 8) {
+    if (kexp) run_diag_exp(desc, nmat, maxRows, mat, kexp, s);
+  }
   if constexpr (sizeof(T) == 4) {
     if (nb == SWEEP_NB_MAX) {
       run_sweep_nb<T, SWEEP_NB_MAX>(desc, nmat, lists, maxRows, maxCols, mat, X, Y, Pbuf, status, tol, s, lo);
@@ -1881,10 +1911,13 @@ static void setup_impl(bddc_ctx* C, cudaStream_t s) {
   //    E = A_II^-1 A_IG and S = A_GG - A_GI E, and E stored over A_IG
   T* const lo[4] = {reinterpret_cast<T*>(C->Xlo.p), reinterpret_cast<T*>(C->Ylo.p),
                     reinterpret_cast<T*>(C->Xlo2.p), reinterpret_cast<T*>(C->Ylo2.p)};
-  run_sweep<T>(C->sw1, nsub, C->gl_sw1, C->maxI, C->maxI, Aloc, Xp, Yp, Pd, status, tol, s, C->nb, lo);
+  run_sweep<T>(C->sw1, nsub, C->gl_sw1, C->maxI, C->maxI, Aloc, Xp, Yp, Pd, status, tol, s, C->kexp.p, C->nb, lo);
   if (C->maxG == 0) return;  // one subdomain: no interface
   launch_list<T, false, false>(C->gl_E, Aloc, Aloc, Et, T(1), T(0), s);
   launch_list<T, false, false>(C->gl_S, Aloc, Et, Aloc, T(-1), T(1), s);
+  if constexpr (sizeof(T) == 8) {
+    if (C->kexp.p) run_diag_exp(C->sgg, nsub, C->maxG, Aloc, C->kexp.p, s);
+  }
   if (C->sparse_cpl) {  // the apply reads the coupling blocks, not E
     if (C->steps_gi > 0) {
       coupling_values_kernel<T><<<cdiv(288 * C->steps_gi, 256), 256, 0, s>>>(
@@ -1919,7 +1952,7 @@ static void setup_impl(bddc_ctx* C, cudaStream_t s) {
     T* const dlo[4] = {reinterpret_cast<T*>(C->DXlo.p), reinterpret_cast<T*>(C->DYlo.p),
                        reinterpret_cast<T*>(C->DXlo2.p), reinterpret_cast<T*>(C->DYlo2.p)};
     run_sweep<T>(C->swd, C->n_dcls, C->gl_swd, C->maxDn, C->maxDn, Dsh, reinterpret_cast<T*>(C->DX.p),
-                 reinterpret_cast<T*>(C->DY.p), reinterpret_cast<T*>(C->DP.p), status, tol, s, C->nb, dlo);
+                 reinterpret_cast<T*>(C->DY.p), reinterpret_cast<T*>(C->DP.p), status, tol, s, C->kexp.p, C->nb, dlo);
     launch_list<T, false, false>(C->gl_dlx, Dsh, Dsb, Ddb, T(1), T(0), s);
     deluxe_transpose_kernel<T><<<gb, 256, 0, s>>>(C->dlx_n.p, C->dlx_ld.p, C->dlx_off.p, Ddb,
                                                         reinterpret_cast<T*>(C->Deb.p));
@@ -1934,7 +1967,7 @@ static void setup_impl(bddc_ctx* C, cudaStream_t s) {
                                           C->cons_idx.p, C->cons_w.p, C->d_offS.p, C->d_ldS.p, Sw);
     CB_LAUNCH();
   }
-  run_sweep<T>(C->sw2, nsub, C->gl_sw2, C->maxG, C->maxG, Sw, Xp, Yp, Pd, status, tol, s, C->nb, lo);
+  run_sweep<T>(C->sw2, nsub, C->gl_sw2, C->maxG, C->maxG, Sw, Xp, Yp, Pd, status, tol, s, C->kexp.p, C->nb, lo);
   // 4. average constraints
   if (C->maxA > 0) {
     cons_y_kernel<T><<<dim3(cdiv(C->maxR, 8), nsub), 256, 0, s>>>(
@@ -1949,7 +1982,7 @@ static void setup_impl(bddc_ctx* C, cudaStream_t s) {
         C->d_na.p, C->d_offCon.p, C->cons_ptr.p, C->cons_idx.p, C->cons_w.p, C->d_offY.p, C->d_ldY.p,
         C->d_offG.p, C->d_ldG.p, Y, G);
     CB_LAUNCH();
-    run_sweep<T>(C->swg, nsub, C->gl_swg, C->maxA, C->maxA, G, Xp, Yp, Pd, status, tol, s, C->nb, lo);
+    run_sweep<T>(C->swg, nsub, C->gl_swg, C->maxA, C->maxA, G, Xp, Yp, Pd, status, tol, s, C->kexp.p, C->nb, lo);
     launch_list<T, false, false>(C->gl_W, G, Zf, Wf, T(1), T(0), s);
     launch_list<T, false, false>(C->gl_T, Y, Wf, Sw, T(-1), T(1), s);
     launch_list<T, false, false>(C->gl_PhiA, Y, G, Phi, T(1), T(0), s);
@@ -2001,7 +2034,7 @@ static void setup_impl(bddc_ctx* C, cudaStream_t s) {
           C->ce_key.p, C->ce_ptr.p, C->ce_src.p, C->n_ce, reinterpret_cast<const double*>(Kc), C->Sc.p);
     CB_LAUNCH();
     run_sweep<double>(C->swc, 1, C->gl_swc, C->n_pi, C->n_pi, C->Sc.p, C->ScX.p, C->ScY.p, C->ScP.p,
-                      status, tol, s);
+                      status, tol, s, C->kexp.p);
     timer_end(CBDDC_TIMER_COARSE_SETUP, s, 2.0 * (double)C->n_pi * C->n_pi * C->n_pi, 0.0);
   }
 }

@@ -32,6 +32,7 @@ struct bddc_ctx {
   cbddc::DVec<unsigned char> Aloc, Sw, Phi, Y, Zf, Wf, G, SPhi, Kc, Xp, Yp, Pd, Et;
   cbddc::DVec<float> tc_scratch;            // split operands of the tensor-core GEMMs (FP32)
   cbddc::DVec<unsigned char> oz_scratch;    // digits of the FP64 tensor-core GEMMs
+  cbddc::DVec<int> kexp;                    // exponents of the diagonals that scale them along K
   cbddc::DVec<float> Xlo, Ylo, DXlo, DYlo;  // second TF32 parts of the sweep panels (FP32)
   cbddc::DVec<float> Xlo2, Ylo2, DXlo2, DYlo2;  // third parts (three-part split)
   int tc_parts_sweep = 0, tc_parts_other = 0;  // TF32 parts per operand chosen at creation
@@ -64,7 +65,7 @@ struct bddc_ctx {
   // apply work vectors
   cbddc::DVec<double> u0, hG, gI, wG, cl, rc, uc, yG, xI, zl;
   // sweep descriptors and GEMM problem lists
-  cbddc::DVec<cbddc::SweepDesc> sw1, sw2, swg, swc;
+  cbddc::DVec<cbddc::SweepDesc> sw1, sw2, swg, swc, sgg;
   int steps1 = 0, steps2 = 0, stepsg = 0, stepsc = 0;
   std::vector<cbddc::GemmList> gl_sw1, gl_sw2, gl_swg, gl_swc;
   cbddc::GemmList gl_E, gl_S, gl_W, gl_T, gl_PhiA, gl_SPhi, gl_Kc;

@@ -31,6 +31,10 @@ struct GemmProb {
   int M, N, K;
   int lda, ldb, ldc;
   int64_t a, b, c;  // element offsets from the kernel's base pointers
+  // FP64 products by integer slices: column k of op(A) is scaled by 2^(ks
+  // kexp[ke + k]) and row k of op(B) by its inverse (0: no scaling)
+  int ks = 0;
+  int64_t ke = 0;
 };
 
 // FP32 setup GEMMs run on the tensor cores (tcgen05, split TF32) unless
@@ -329,6 +333,7 @@ struct GemmList {
   std::vector<oz::Batch> oz_batches;
   unsigned char* oz_base = nullptr;
   int* oz_status = nullptr;
+  const int* oz_kexp = nullptr;  // exponents along K
   std::unique_ptr<GemmList> panel;  // FP64 sweep step: Y = P A_kk as products of their own
   // order 1: tiles of the largest problems (M N K) first, so that with
   // uneven subdomains the long tile runs of a persistent kernel start early
@@ -382,7 +387,7 @@ struct GemmList {
       const GemmProb& q = v[i];
       if (q.M <= 0 || q.N <= 0 || q.K <= 0) {
         pr[i] = oz::Prob{0, 0, 0, 0, 0, 0, 0};
-        sa[i] = sb[i] = oz::SplitProb{0, 0, 0, 0, 0};
+        sa[i] = sb[i] = oz::SplitProb{0, 0, 0, 0, 0, 0, 0};
         continue;
       }
       CB_CHECK(q.K <= 1 << 24, CBDDC_EINVAL, "dense product too long");
@@ -406,8 +411,8 @@ struct GemmList {
       oz::Batch& b = oz_batches.back();
       b.Kp = std::max(b.Kp, Kp);
       pr[i] = oz::Prob{q.M, q.N, q.K, q.ldc, q.c, (int)b.rowsA, (int)b.rowsB};
-      sa[i] = oz::SplitProb{q.M, q.K, q.lda, (int)b.rowsA, q.a};
-      sb[i] = oz::SplitProb{q.N, q.K, q.ldb, (int)b.rowsB, q.b};
+      sa[i] = oz::SplitProb{q.M, q.K, q.lda, (int)b.rowsA, q.ks, q.a, q.ke};
+      sb[i] = oz::SplitProb{q.N, q.K, q.ldb, (int)b.rowsB, -q.ks, q.b, q.ke};
       b.rowsA += q.M;
       b.rowsB += q.N;
       for (int k = 0; k < (int)cdiv(q.M, 32); ++k) ia.push_back(make_int2(i, k));
@@ -429,9 +434,10 @@ struct GemmList {
     for (const auto& b : oz_batches) m = std::max(m, b.bytes());
     return m;
   }
-  void bind_oz(unsigned char* base, int* status) {
+  void bind_oz(unsigned char* base, int* status, const int* kexp = nullptr) {
     oz_base = base;
     oz_status = status;
+    oz_kexp = kexp;
     for (auto& b : oz_batches) {
       b.maps.a = oz::encode_digits(reinterpret_cast<__half*>(base), b.rowsA, b.Kp, oz::BM);
       b.maps.b = oz::encode_digits(reinterpret_cast<__half*>(base + b.bytes_a()), b.rowsB, b.Kp, oz::BN);
@@ -564,9 +570,9 @@ void launch_oz(const GemmList& g, const double* A, const double* B, double* C, d
     __half* db = reinterpret_cast<__half*>(g.oz_base + b.bytes_a());
     int* ea = reinterpret_cast<int*>(g.oz_base + b.bytes_a() + b.bytes_b());
     int* eb = reinterpret_cast<int*>(g.oz_base + b.bytes_a() + b.bytes_b() + b.bytes_ea());
-    oz::split_kernel<!TA><<<b.na, 256, 0, s>>>(g.oz_ia.p + b.a0, g.oza.p, b.Kp, A, da, b.rowsA * b.Kp, ea);
+    oz::split_kernel<!TA><<<b.na, 256, 0, s>>>(g.oz_ia.p + b.a0, g.oza.p, b.Kp, A, g.oz_kexp, da, b.rowsA * b.Kp, ea);
     CB_LAUNCH();
-    oz::split_kernel<TB><<<b.nb, 256, 0, s>>>(g.oz_ib.p + b.b0, g.ozb.p, b.Kp, B, db, b.rowsB * b.Kp, eb);
+    oz::split_kernel<TB><<<b.nb, 256, 0, s>>>(g.oz_ib.p + b.b0, g.ozb.p, b.Kp, B, g.oz_kexp, db, b.rowsB * b.Kp, eb);
     CB_LAUNCH();
     const int grid = tc::tc_grid(b.nt);
     if (beta == 0.0)
@@ -632,7 +638,20 @@ struct SweepDesc {
   int64_t offX;           // X panel offset (rows x NB, ld NB)
   int64_t offY;           // Y panel offset (NB x cols, ld ld)
   int64_t offP;           // diagonal inverse (NB x NB)
+  int64_t ke = 0;         // FP64: first of its exponents (diag_exp_kernel)
 };
+
+// kexp[ke + i] = half the exponent of diagonal entry i: 2^kexp is the square
+// root of the entry within a factor of two, the Jacobi scaling of row and
+// column i (0 for entries that are zero or not finite).
+static __global__ void diag_exp_kernel(const SweepDesc* __restrict__ desc, const double* __restrict__ mat,
+                                       int* __restrict__ kexp) {
+  const SweepDesc d = desc[blockIdx.y];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= d.rows) return;
+  const int e = oz::exp_key(mat[d.off + (int64_t)i * d.ld + i]);
+  kexp[d.ke + i] = e == 0 || e == 2047 ? 0 : (e - 1023) >> 1;
+}
 
 // P = inverse of the kb x kb diagonal block of pivot step k, by Gauss-Jordan
 // in the operator precision T: at pivot j
