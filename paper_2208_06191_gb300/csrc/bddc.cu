@@ -1767,12 +1767,8 @@ template <typename T, int NB, int NP, int CH>
 static void panel_launch_ch(int n, int nmat, cudaStream_t s, const SweepDesc* desc, int k, T* mat, const T* Pbuf,
                             T* X, T* Y, T* const* lo) {
   constexpr size_t smem = NP < 0 ? 0 : panel_smem_bytes<T, NB, CH>();
-  static bool attr = false;
-  if (!attr) {
-    CB_CUDA(cudaFuncSetAttribute(sweep_panel_kernel<T, NB, NP, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    attr = true;
-  }
+  static PerDevice<bool> done;
+  allow_smem(done, sweep_panel_kernel<T, NB, NP, CH>, smem);
   sweep_panel_kernel<T, NB, NP, CH><<<dim3(cdiv(n, CH), nmat), 256, smem, s>>>(desc, k, mat, Pbuf, X, Y, lo[0],
                                                                               lo[1], lo[2], lo[3]);
   CB_LAUNCH();

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/cardiac_bddc.h"
+#include "per_device.h"
 
 namespace cbddc {
 
@@ -34,6 +35,23 @@ void set_last_error(const std::string& msg);
   do {                                                                       \
     if (!(cond)) throw ::cbddc::Error{(code), (msg)};                        \
   } while (0)
+
+inline int current_device() {
+  int dev = 0;
+  CB_CUDA(cudaGetDevice(&dev));
+  return dev;
+}
+
+// Lets a kernel use up to bytes of dynamic shared memory.  The attribute
+// belongs to the function on the current device, so done (a static of the
+// caller, one per kernel) remembers the devices.
+template <typename K>
+inline void allow_smem(PerDevice<bool>& done, K* kernel, size_t bytes) {
+  done.get(current_device(), [&] {
+    CB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return true;
+  });
+}
 
 // Counts every kernel launch of the library and checks the launch status.
 void count_launch();

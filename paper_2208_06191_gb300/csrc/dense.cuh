@@ -534,7 +534,6 @@ void launch_tc(const GemmList& g, const float* A, const float* B, float* C, floa
     }
     CB_LAUNCH();
   }
-  tc::set_smem_attr();
   // rank-64 sweep updates (two K chunks) are bound by C's traffic: one
   // operand stage and two C buffers; longer K: two stages and one C buffer
   // (three-part operands: one stage and two C buffers always)
@@ -542,6 +541,7 @@ void launch_tc(const GemmList& g, const float* A, const float* B, float* C, floa
   // one K-step per TMEM slice (else a 32-wide K block per slice)
   const bool ks1 = g.presplit ? tc_sweep_ks1() : tc_other_ks1();
 #define CB_TC_LAUNCH(NST, NCB, NP, KS)                                                              \
+  tc::set_smem_attr<NST, NCB, NP, KS>(),                                                            \
   tc::tc_gemm_kernel<NST, NCB, NP, KS><<<grid, tc::TC_THREADS, tc::TcSmem<NST, NCB, NP>::bytes, s>>>( \
       g.tiles.p, g.ntiles, g.tcp.p, g.maps, C, alpha, beta, g.tc_status)
   if (g.np == 3) {
@@ -564,7 +564,6 @@ template <bool TA, bool TB>
 void launch_oz(const GemmList& g, const double* A, const double* B, double* C, double alpha, double beta,
                cudaStream_t s) {
   CB_CHECK((alpha == 1.0 || alpha == -1.0) && (beta == 0.0 || beta == 1.0), CBDDC_EINVAL, "dense product factors");
-  oz::set_smem_attr();
   for (const oz::Batch& b : g.oz_batches) {
     __half* da = reinterpret_cast<__half*>(g.oz_base);
     __half* db = reinterpret_cast<__half*>(g.oz_base + b.bytes_a());
@@ -575,6 +574,8 @@ void launch_oz(const GemmList& g, const double* A, const double* B, double* C, d
     oz::split_kernel<TB><<<b.nb, 256, 0, s>>>(g.oz_ib.p + b.b0, g.ozb.p, b.Kp, B, g.oz_kexp, db, b.rowsB * b.Kp, eb);
     CB_LAUNCH();
     const int grid = tc::tc_grid(b.nt);
+    if (beta == 0.0) oz::set_smem_attr<false>();
+    else oz::set_smem_attr<true>();
     if (beta == 0.0)
       oz::gemm_kernel<false><<<grid, oz::THREADS, oz::SMEM, s>>>(g.oz_tiles.p + b.t0, b.nt, g.ozp.p, b.maps, ea, eb,
                                                                  C, alpha < 0.0, g.oz_status);

@@ -1148,12 +1148,8 @@ void assemble(fem_problem* P, const double* d, double lam, double* residual, boo
     hex2_element_kernel<false><<<cdiv(P->n_el, H2_WARPS), 32 * H2_WARPS, 0, s>>>(
         mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, nullptr, P->status.p, P->n_el);
   } else {
-    static bool attr = false;
-    if (!attr) {
-      CB_CUDA(cudaFuncSetAttribute(hex2_element_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)H2T_SMEM));
-      attr = true;
-    }
+    static PerDevice<bool> done;
+    allow_smem(done, hex2_element_kernel<true>, H2T_SMEM);
     hex2_element_kernel<true><<<cdiv(P->n_el, H2T_WARPS), 32 * H2T_WARPS, H2T_SMEM, s>>>(
         mp, P->elems.p, P->hex2_geo.p, P->d_full.p, accf, P->rcontrib.p, P->contrib.p, P->status.p, P->n_el);
   }

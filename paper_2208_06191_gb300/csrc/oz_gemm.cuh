@@ -557,12 +557,10 @@ struct Batch {
 // batch of its own.
 constexpr int64_t kBatchBytes = (int64_t)2 << 30;
 
+template <bool ADD>
 inline void set_smem_attr() {
-  static bool done = false;
-  if (done) return;
-  CB_CUDA(cudaFuncSetAttribute(gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-  CB_CUDA(cudaFuncSetAttribute(gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-  done = true;
+  static PerDevice<bool> done;
+  allow_smem(done, gemm_kernel<ADD>, SMEM);
 }
 
 }  // namespace oz

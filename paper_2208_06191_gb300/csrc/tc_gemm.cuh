@@ -567,15 +567,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 inline EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
+  static const EncodeTiledFn fn = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     CB_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q));
     CB_CHECK(q == cudaDriverEntryPointSuccess && p != nullptr, CBDDC_ECUDA,
              "cuTensorMapEncodeTiled is not available from the driver");
-    fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+    return reinterpret_cast<EncodeTiledFn>(p);
+  }();
   return fn;
 }
 
@@ -597,33 +596,21 @@ inline CUtensorMap encode_kmajor(const float* base, int64_t rows, int Kp) {
 }
 
 template <int NST, int NCB, int NP, int KS>
-inline void set_smem_attr_one() {
-  CB_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<NST, NCB, NP, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TcSmem<NST, NCB, NP>::bytes));
-}
-
 inline void set_smem_attr() {
-  static bool done = false;
-  if (!done) {
-    set_smem_attr_one<1, 2, 2, 1>();
-    set_smem_attr_one<1, 2, 2, 4>();
-    set_smem_attr_one<2, 1, 2, 4>();
-    set_smem_attr_one<2, 1, 2, 1>();
-    set_smem_attr_one<1, 2, 3, 1>();
-    set_smem_attr_one<1, 2, 3, 4>();
-    done = true;
-  }
+  static PerDevice<bool> done;
+  allow_smem(done, tc_gemm_kernel<NST, NCB, NP, KS>, TcSmem<NST, NCB, NP>::bytes);
 }
 
 // Persistent CTAs: one per SM (one fits), never more than tiles.
 inline int tc_grid(int ntiles) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    CB_CUDA(cudaGetDevice(&dev));
-    CB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return std::max(1, std::min(ntiles, sms));
+  static PerDevice<int> sms;
+  const int dev = current_device();
+  const int n = sms.get(dev, [&] {
+    int v = 0;
+    CB_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
+    return v;
+  });
+  return std::max(1, std::min(ntiles, n));
 }
 
 }  // namespace tc
