@@ -44,7 +44,9 @@ inline int current_device() {
 
 // Lets a kernel use up to bytes of dynamic shared memory.  The attribute
 // belongs to the function on the current device, so done (a static of the
-// caller, one per kernel) remembers the devices.
+// caller, one per kernel) remembers the devices.  The caller has internal linkage:
+// the statics of inline functions are one object for all libraries of a process,
+// but each library has kernels of its own.
 template <typename K>
 inline void allow_smem(PerDevice<bool>& done, K* kernel, size_t bytes) {
   done.get(current_device(), [&] {

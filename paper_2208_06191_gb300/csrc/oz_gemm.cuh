@@ -558,7 +558,7 @@ struct Batch {
 constexpr int64_t kBatchBytes = (int64_t)2 << 30;
 
 template <bool ADD>
-inline void set_smem_attr() {
+static void set_smem_attr() {
   static PerDevice<bool> done;
   allow_smem(done, gemm_kernel<ADD>, SMEM);
 }

@@ -596,7 +596,7 @@ inline CUtensorMap encode_kmajor(const float* base, int64_t rows, int Kp) {
 }
 
 template <int NST, int NCB, int NP, int KS>
-inline void set_smem_attr() {
+static void set_smem_attr() {
   static PerDevice<bool> done;
   allow_smem(done, tc_gemm_kernel<NST, NCB, NP, KS>, TcSmem<NST, NCB, NP>::bytes);
 }
