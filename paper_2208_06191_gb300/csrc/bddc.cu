@@ -1495,7 +1495,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       gPV.push_back(GemmProb{C->nr[s], C->nv[s], C->nr[s], C->ldS[s], C->ldA[s], C->ldPhi[s], C->offS[s],
                              aGG + (int64_t)C->nr[s] * C->ldA[s], C->offPhi[s], 1, sgg[s].ke});
     }
-    C->gl_PsiV.set(gPV, es, true, C->tile_order);
+    C->gl_PsiV.set(gPV, es, true, C->tile_order, true);
     C->Psi.alloc(sized(C->offPhi[nsub]));
   }
 
@@ -1707,9 +1707,20 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
         }
     }
     int64_t need = 0;
-    for (auto* g : lists) need = std::max(need, g->oz_bytes());
+    for (int64_t cap = oz::kBatchBytes;;) {
+      need = 0;
+      for (auto* g : lists) need = std::max(need, g->oz_bytes());
+      try {
+        C->oz_scratch.alloc((size_t)need);
+        break;
+      } catch (const Error& e) {
+        if (e.code != CBDDC_ENOMEM || cap <= oz::kMinBatchBytes) throw;
+      }
+      cap = std::max(cap / 4, oz::kMinBatchBytes);
+      for (auto* g : lists)
+        if (g->ntiles > 0) g->plan_oz(cap);
+    }
     if (need > 0) {
-      C->oz_scratch.alloc((size_t)need);
       C->kexp.alloc((size_t)nke);
       for (auto* g : lists) g->bind_oz(C->oz_scratch.p, P->status.p, C->kexp.p);
     }
@@ -2286,14 +2297,24 @@ bddc_ctx::~bddc_ctx() {
 }
 
 int64_t bddc_ctx::device_bytes() const {
-  return (int64_t)(Aloc.bytes() + Sw.bytes() + Phi.bytes() + Y.bytes() + Zf.bytes() + Wf.bytes() +
-                   G.bytes() + SPhi.bytes() + Kc.bytes() + Xp.bytes() + Yp.bytes() + Pd.bytes() + Et.bytes() +
-                   Sc.bytes() + ScX.bytes() + ScY.bytes() + ScP.bytes() + u0.bytes() + hG.bytes() +
-                   gI.bytes() + wG.bytes() + cl.bytes() + rc.bytes() + uc.bytes() + yG.bytes() + gl.bytes() + xI.bytes() + zl.bytes() +
-                   Dsb.bytes() + Ddb.bytes() + Deb.bytes() + Dsh.bytes() + DX.bytes() + DY.bytes() + DP.bytes() +
-                   yD.bytes() + Psi.bytes() + sgi_off.bytes() + sgi_len.bytes() + sgi_row.bytes() +
-                   sgi_col.bytes() + sgi_src.bytes() + sgi_val.bytes() + sig_off.bytes() + sig_len.bytes() +
-                   sig_row.bytes() + sig_col.bytes() + sig_src.bytes() + sig_val.bytes() + uq.bytes() +
-                   zq.bytes()) +
-         (next ? next->device_bytes() + coarse_prob->device_bytes() : 0);
+  int64_t b = 0;
+  auto add = [&](const auto&... v) { ((b += (int64_t)v.bytes()), ...); };
+  auto plans = [&](const auto&... g) { ((b += g.device_bytes()), ...); };
+  add(d_nI, d_nG, d_nr, d_nv, d_na, d_nc, d_ns, d_ldA, d_ldS, d_ldPhi, d_ldY, d_ldG, d_offA, d_offS, d_offPhi, d_offY,
+      d_offZ, d_offG, d_offSPhi, d_offKc, d_offE, d_offI, d_offGam, d_offC, d_offCon, d_offN);
+  add(perm, gdofI, gdofG, Dg, gam_if, if_dof, if_ptr, if_src, cons_ptr, cons_idx, cons_w, gprim, cg_ptr, cg_src, cnch,
+      itI, itG, itP, itR, ce_key, ce_ptr, ce_src, d_cbase);
+  add(Aloc, Sw, Phi, Psi, Y, Zf, Wf, G, SPhi, Kc, Xp, Yp, Pd, Et, Sc, ScX, ScY, ScP, kexp);
+  add(oz_scratch, tc_scratch, Xlo, Ylo, Xlo2, Ylo2, DXlo, DYlo, DXlo2, DYlo2);
+  add(dlx_n, dlx_sub, dlx_ld, dlx_pos, dcls_ptr, dcls_blk, dlx_poff, dlx_off, dcls_off, Dsb, Ddb, Deb, Dsh, DX, DY, DP,
+      yD);
+  add(sgi_off, sgi_len, sgi_row, sgi_col, sgi_src, sgi_val, sig_off, sig_len, sig_row, sig_col, sig_src, sig_val, uq,
+      zq);
+  add(u0, hG, gI, wG, cl, rc, uc, yG, xI, zl, gl, sw1, sw2, swg, swc, sgg, swd);
+  add(gm.V, gm.Zb, gm.w, gm.r, gm.H, gm.cs, gm.sn, gm.g, gm.y, gm.h, gm.partial, gm.scal, gm.ticket, gm.cpart,
+      gm.mpart, nw_r, nw_b, nw_delta, nw_d);
+  plans(gl_E, gl_S, gl_W, gl_T, gl_PhiA, gl_SPhi, gl_Kc, gl_PsiV, gl_dlx);
+  for (const auto* v : {&gl_sw1, &gl_sw2, &gl_swg, &gl_swc, &gl_swd})
+    for (const auto& g : *v) plans(g);
+  return b + (next ? next->device_bytes() + coarse_prob->device_bytes() : 0);
 }

@@ -101,6 +101,7 @@ struct DVec {
     cudaError_t e = cudaMalloc(&p, count * sizeof(T));
     if (e != cudaSuccess) {
       p = nullptr;
+      (void)cudaGetLastError();  // reported here, not at the next launch
       throw Error{CBDDC_ENOMEM, "cudaMalloc of " + std::to_string(count * sizeof(T)) +
                                     " bytes failed: " + cudaGetErrorString(e)};
     }

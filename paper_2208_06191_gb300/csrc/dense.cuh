@@ -335,10 +335,15 @@ struct GemmList {
   int* oz_status = nullptr;
   const int* oz_kexp = nullptr;  // exponents along K
   std::unique_ptr<GemmList> panel;  // FP64 sweep step: Y = P A_kk as products of their own
+  bool trans_a = false, trans_b = false;
+  int tile_order = 0;
   // order 1: tiles of the largest problems (M N K) first, so that with
   // uneven subdomains the long tile runs of a persistent kernel start early
-  void set(const std::vector<GemmProb>& v, size_t esize, bool ta = false, int order = 0) {
+  void set(const std::vector<GemmProb>& v, size_t esize, bool ta = false, int order = 0, bool tb = false) {
     h = v;
+    trans_a = ta;
+    trans_b = tb;
+    tile_order = order;
     n = (int)v.size();
     flops = bytes = 0.0;
     const int w = (int)(16 / esize);
@@ -363,62 +368,73 @@ struct GemmList {
     tiles.upload(t);
     tc_planned = tc_bound = false;
     if (esize == 4 && ntiles > 0 && n <= 65535) plan_tc(v);
-    if (esize == 8 && ntiles > 0) plan_oz(v, order);
+    if (esize == 8 && ntiles > 0) plan_oz();
   }
-  // FP64: batches of problems whose digits share the scratch buffer, with
-  // the split work items (blocks of 32 rows) and the output tiles of each
-  void plan_oz(const std::vector<GemmProb>& v, int order) {
-    std::vector<oz::Prob> pr(n);
-    std::vector<oz::SplitProb> sa(n), sb(n);
+  // FP64: batches of problems, or of blocks of whole tiles of a problem, whose
+  // digits share a buffer of cap bytes (one tile row and column fit whatever the
+  // cap), with the split work items (blocks of 32 rows) and the output tiles of
+  // each
+  void plan_oz(int64_t cap = oz::kBatchBytes) {
+    std::vector<oz::Prob> pr;
+    std::vector<oz::SplitProb> sa, sb;
     std::vector<int2> ia, ib;
     std::vector<int4> t;
     oz_batches.clear();
-    auto work = [&](const int4& a) { return (double)v[a.x].M * v[a.x].N * v[a.x].K; };
+    auto work = [&](const int4& a) { return (double)pr[a.x].M * pr[a.x].N * pr[a.x].K; };
     auto close = [&] {
       if (oz_batches.empty()) return;
       oz::Batch& b = oz_batches.back();
       b.na = (int)ia.size() - b.a0;
       b.nb = (int)ib.size() - b.b0;
       b.nt = (int)t.size() - b.t0;
-      if (order == 1)
+      if (tile_order == 1)
         std::stable_sort(t.begin() + b.t0, t.end(), [&](const int4& x, const int4& y) { return work(x) > work(y); });
     };
-    for (int i = 0; i < n; ++i) {
-      const GemmProb& q = v[i];
-      if (q.M <= 0 || q.N <= 0 || q.K <= 0) {
-        pr[i] = oz::Prob{0, 0, 0, 0, 0, 0, 0};
-        sa[i] = sb[i] = oz::SplitProb{0, 0, 0, 0, 0, 0, 0};
-        continue;
-      }
+    for (const GemmProb& q : h) {
+      if (q.M <= 0 || q.N <= 0 || q.K <= 0) continue;
       CB_CHECK(q.K <= 1 << 24, CBDDC_EINVAL, "dense product too long");
       const int Kp = (int)round_up(q.K, oz::BK);
-      bool fresh = oz_batches.empty();
-      if (!fresh) {
-        oz::Batch b = oz_batches.back();
-        b.Kp = std::max(b.Kp, Kp);
-        b.rowsA += q.M;
-        b.rowsB += q.N;
-        fresh = b.bytes() > oz::kBatchBytes || b.rowsA >= INT32_MAX || b.rowsB >= INT32_MAX;
+      // rows of op(A) and columns of op(B) per block: all of them, or as many
+      // rows as fit beside all columns, or half of the cap each
+      const int64_t fit = cap / ((int64_t)oz::S * Kp * 2 + 8);
+      int bm = q.M, bn = q.N;
+      if ((int64_t)q.M + q.N > fit) {
+        if (q.N > fit / 2) bn = (int)std::min<int64_t>(q.N, std::max<int64_t>(oz::BN, fit / 2 / oz::BN * oz::BN));
+        bm = (int)std::min<int64_t>(q.M, std::max<int64_t>(oz::BM, (fit - bn) / oz::BM * oz::BM));
       }
-      if (fresh) {
-        close();
-        oz::Batch b;
-        b.a0 = (int)ia.size();
-        b.b0 = (int)ib.size();
-        b.t0 = (int)t.size();
-        oz_batches.push_back(b);
-      }
-      oz::Batch& b = oz_batches.back();
-      b.Kp = std::max(b.Kp, Kp);
-      pr[i] = oz::Prob{q.M, q.N, q.K, q.ldc, q.c, (int)b.rowsA, (int)b.rowsB};
-      sa[i] = oz::SplitProb{q.M, q.K, q.lda, (int)b.rowsA, q.ks, q.a, q.ke};
-      sb[i] = oz::SplitProb{q.N, q.K, q.ldb, (int)b.rowsB, -q.ks, q.b, q.ke};
-      b.rowsA += q.M;
-      b.rowsB += q.N;
-      for (int k = 0; k < (int)cdiv(q.M, 32); ++k) ia.push_back(make_int2(i, k));
-      for (int k = 0; k < (int)cdiv(q.N, 32); ++k) ib.push_back(make_int2(i, k));
-      for (int tm = 0; tm < (int)cdiv(q.M, oz::BM); ++tm)
-        for (int tn = 0; tn < (int)cdiv(q.N, oz::BN); ++tn) t.push_back(make_int4(i, tm, tn, 0));
+      for (int m0 = 0; m0 < q.M; m0 += bm)
+        for (int n0 = 0; n0 < q.N; n0 += bn) {
+          const int M = std::min(bm, q.M - m0), N = std::min(bn, q.N - n0), i = (int)pr.size();
+          bool fresh = oz_batches.empty();
+          if (!fresh) {
+            oz::Batch b = oz_batches.back();
+            b.Kp = std::max(b.Kp, Kp);
+            b.rowsA += M;
+            b.rowsB += N;
+            fresh = b.bytes() > cap || b.rowsA >= INT32_MAX || b.rowsB >= INT32_MAX;
+          }
+          if (fresh) {
+            close();
+            oz::Batch b;
+            b.a0 = (int)ia.size();
+            b.b0 = (int)ib.size();
+            b.t0 = (int)t.size();
+            oz_batches.push_back(b);
+          }
+          oz::Batch& b = oz_batches.back();
+          b.Kp = std::max(b.Kp, Kp);
+          pr.push_back(oz::Prob{M, N, q.K, q.ldc, q.c + (int64_t)m0 * q.ldc + n0, (int)b.rowsA, (int)b.rowsB});
+          sa.push_back(oz::SplitProb{M, q.K, q.lda, (int)b.rowsA, q.ks, q.a + (int64_t)m0 * (trans_a ? 1 : q.lda),
+                                     q.ke});
+          sb.push_back(oz::SplitProb{N, q.K, q.ldb, (int)b.rowsB, -q.ks, q.b + (int64_t)n0 * (trans_b ? q.ldb : 1),
+                                     q.ke});
+          b.rowsA += M;
+          b.rowsB += N;
+          for (int k = 0; k < (int)cdiv(M, 32); ++k) ia.push_back(make_int2(i, k));
+          for (int k = 0; k < (int)cdiv(N, 32); ++k) ib.push_back(make_int2(i, k));
+          for (int tm = 0; tm < (int)cdiv(M, oz::BM); ++tm)
+            for (int tn = 0; tn < (int)cdiv(N, oz::BN); ++tn) t.push_back(make_int4(i, tm, tn, 0));
+        }
     }
     close();
     ozp.upload(pr);
@@ -427,6 +443,12 @@ struct GemmList {
     oz_ia.upload(ia);
     oz_ib.upload(ib);
     oz_tiles.upload(t);
+  }
+  // device memory of the plan itself
+  int64_t device_bytes() const {
+    return (int64_t)(d.bytes() + tiles.bytes() + tcp.bytes() + spa.bytes() + spb.bytes() + ozp.bytes() + oza.bytes() +
+                     ozb.bytes() + oz_ia.bytes() + oz_ib.bytes() + oz_tiles.bytes()) +
+           (panel ? panel->device_bytes() : 0);
   }
   // bytes of digit scratch this list needs
   int64_t oz_bytes() const {

@@ -455,7 +455,8 @@ gemm_kernel(const int4* __restrict__ tiles, int ntiles, const Prob* __restrict__
       int top = 0;
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
-        const int h = (int)(hi[q] >> 32);
+        // (columns past N hold products with another problem's digits)
+        const int h = n0 + q < p.N ? (int)(hi[q] >> 32) : 0;
         top |= h ^ (h >> 31);
       }
       const int sh = max(0, 64 - 35 - __clz(top));
@@ -553,9 +554,14 @@ struct Batch {
   int64_t bytes() const { return bytes_a() + bytes_b() + bytes_ea() + round_up(rowsB * 4, 256); }
 };
 
-// Problems share a batch while its digits fit this; a larger problem gets a
-// batch of its own.
-constexpr int64_t kBatchBytes = (int64_t)2 << 30;
+// Digits of one batch, at most: problems share a batch while they fit, and
+// a larger one is cut into blocks of whole tiles.  A context keeps one buffer of
+// this size, or less where its products need less or the memory is short (down
+// to the second figure).  Each batch costs three launches and a last wave of
+// tiles: the FP64 Newton step of the 48x48x12 slab (60 ms), whose E and S take 2.3
+// and 2.4 GB of digits, takes 1% longer with 1 GiB than with 2 GiB, and 2% longer
+// with 512 MiB.
+constexpr int64_t kBatchBytes = (int64_t)1 << 30, kMinBatchBytes = (int64_t)8 << 20;
 
 template <bool ADD>
 static void set_smem_attr() {
