@@ -440,13 +440,21 @@ enum {
                                  Gauss-Jordan sweeps and the E, S, constraint
                                  and coarse-basis products (tensor cores)     */
   CBDDC_TIMER_ELEMENT = 2,    /* element residual/tangent kernel              */
-  CBDDC_TIMER_APPLY = 3,      /* one whole BDDC apply (all its launches)      */
+  CBDDC_TIMER_APPLY = 3,      /* one whole BDDC apply (all its launches);
+                                 GMRES runs one apply and one SpMV more than
+                                 it has iterations where it had launched a
+                                 step before the last residual was known      */
   CBDDC_TIMER_SPMV = 4,       /* BSR SpMV                                     */
   CBDDC_TIMER_ORTH = 5,       /* one GMRES Arnoldi step (Gram-Schmidt,
-                                 Givens, normalisation)                       */
+                                 Givens, normalisation); one per iteration    */
   CBDDC_TIMER_SETUP = 6,      /* one whole BDDC setup (all levels)            */
   CBDDC_TIMER_LEVEL2_SETUP = 7, /* setup of the level-2 BDDC (multilevel)     */
-  CBDDC_TIMER_LEVEL2_APPLY = 8, /* apply of the level-2 BDDC (multilevel)     */
+  CBDDC_TIMER_LEVEL2_APPLY = 8, /* apply of the level-2 BDDC (multilevel).
+                                   While this class or COARSE_APPLY is
+                                   recorded, the coarse correction of the
+                                   apply runs before the local solves and not
+                                   beside them, so that these times are parts
+                                   of APPLY's, which is longer by them        */
   CBDDC_TIMER_COARSE_SETUP = 9, /* coarsest level: FP64 coarse assembly and
                                    dense inverse                              */
   CBDDC_TIMER_COARSE_APPLY = 10, /* coarsest level: dense FP64 coarse solve   */

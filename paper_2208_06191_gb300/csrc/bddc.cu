@@ -2109,8 +2109,11 @@ void apply_with_work(bddc_ctx* C, const double* r, double* z, const ApplyWork& w
     // T g are independent until the prolongation.  The coarse chain is short
     // kernels that leave the GPU mostly idle (48x48x12 slab: 33 us beside the
     // 46 us of T g; three levels: the whole level-2 apply), so it runs on the
-    // context's second stream between two events of the caller's.
-    const bool fork = C->n_pi > 0 && C->n_itG > 0;
+    // context's second stream between two events of the caller's.  While its own
+    // time is recorded it stays on the caller's stream, so that it is a part of
+    // the apply's time and not beside the rest of it.
+    const bool fork = C->n_pi > 0 && C->n_itG > 0 && !timer_active(CBDDC_TIMER_LEVEL2_APPLY) &&
+                      !timer_active(CBDDC_TIMER_COARSE_APPLY);
     cudaStream_t sc = s;
     if (fork) {
       sc = C->side;

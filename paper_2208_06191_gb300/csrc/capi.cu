@@ -45,11 +45,13 @@ struct ClassTimer {
   bool open = false;  // the outermost begin recorded an event
   int64_t launches = 0;
   double flops = 0.0, bytes = 0.0;
+  bool last = false;  // the last begin/end pair was recorded, with these flops and bytes
+  double last_flops = 0.0, last_bytes = 0.0;
   static constexpr size_t kMax = 65536;
   void reset() {
     used = 0;
     depth = 0;
-    open = false;
+    open = last = false;
     launches = 0;
     flops = bytes = 0.0;
   }
@@ -84,13 +86,29 @@ void timer_end(int kernel_class, cudaStream_t s, double flops, double bytes) {
   if (!timer_active(kernel_class)) return;
   ClassTimer& t = g_timers[kernel_class];
   if (t.depth == 0) return;
-  if (--t.depth > 0 || !t.open) return;
+  if (--t.depth > 0) return;
+  t.last = t.open;
+  t.last_flops = flops;
+  t.last_bytes = bytes;
+  if (!t.open) return;
   CB_CUDA(cudaEventRecord(t.pool[t.used + 1], s));
   t.open = false;
   t.used += 2;
   t.launches += 1;
   t.flops += flops;
   t.bytes += bytes;
+}
+
+// The last recorded launch of a class turned out to have done nothing.
+void timer_drop(int kernel_class) {
+  if (!timer_active(kernel_class)) return;
+  ClassTimer& t = g_timers[kernel_class];
+  if (!t.last) return;
+  t.used -= 2;
+  t.launches -= 1;
+  t.flops -= t.last_flops;
+  t.bytes -= t.last_bytes;
+  t.last = false;
 }
 
 static void timer_totals(int kernel_class, double* total_ms, int64_t* launches, double* flops, double* bytes) {

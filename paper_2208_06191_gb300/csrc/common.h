@@ -67,6 +67,7 @@ void count_launch();
 bool timer_active(int kernel_class);
 void timer_begin(int kernel_class, cudaStream_t s);
 void timer_end(int kernel_class, cudaStream_t s, double flops, double bytes);
+void timer_drop(int kernel_class);  // forgets the class's last launch
 
 // Device-side error bits, OR-ed into a status word by kernels.
 enum : int {

@@ -937,7 +937,11 @@ int gmres_run(fem_problem* P, bddc_ctx* C, Gmres& G, const double* b, double* x,
       std::memcpy(flags, slot + 8, sizeof flags);
       res = slot[0];
       ++total;
-      if (flags[0]) break;
+      if (flags[0]) {
+        // (its product and preconditioner ran, its Gram-Schmidt step did not)
+        if (launched > j + 1) timer_drop(CBDDC_TIMER_ORTH);
+        break;
+      }
     }
     // x += Z y over the columns built in this cycle
     backsolve_kernel<<<1, 256, 0, s>>>(G.H.p, m, kcount, G.g.p, G.y.p);
