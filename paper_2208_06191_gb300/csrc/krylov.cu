@@ -247,8 +247,8 @@ __global__ void givens_kernel(int j, int m, double* __restrict__ H, double* __re
 // is issued beside the FMAs: dots take eight columns per warp and a segment of
 // the rows, and reduce the eight sums together at the end of the chunk (9
 // additions instead of 40); updates take 32 rows and a part of the columns per
-// warp.  The second phase goes through the chunk in tiles, update then dots,
-// so that the dots find the tile's part of V in the cache.  After each barrier
+// warp, two to four parts so that the 16 warps have about 64 of these shares (a
+// chunk has at most 1024 rows on 152 SMs), added at the end.  After each barrier
 // every CTA sums all CTAs' partials in CTA order (identical on every CTA,
 // independent of scheduling).
 // Mean Arnoldi step of a solve: 60 us at n = 86k and 59 vectors (100 us with
@@ -256,8 +256,7 @@ __global__ void givens_kernel(int j, int m, double* __restrict__ H, double* __re
 // chain on global memory), 51 us at n = 27k and 90 vectors (114 us).
 constexpr int CGS_THREADS = 512;
 constexpr int CGS_WARPS = CGS_THREADS / 32;
-constexpr int CGS_JS = 4;  // column parts of the update, at most
-constexpr int CGS_TILE = 32 * CGS_WARPS;  // rows of a tile (one 32-row block per warp)
+constexpr int CGS_JS = 4;  // column parts of the update, at most (two at least)
 struct CgsArgs {
   const double* V;   // nvec columns of length n (stride n)
   int64_t n;
@@ -289,15 +288,15 @@ struct CgsDots {
 #pragma unroll
     for (int q = 0; q < 8; ++q) s[q] = 0.0;
   }
-  // rows [t0, t1) of the chunk (t0 a multiple of 32)
-  __device__ void add(const CgsArgs& a, const double* __restrict__ ws, int64_t r0, int t0, int t1) {
+  // the rows of the chunk
+  __device__ void add(const CgsArgs& a, const double* __restrict__ ws, int64_t r0, int rows) {
     if (!active) return;
     const int lane = threadIdx.x & 31;
     const double* p[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) p[q] = a.V + (int64_t)min(c0 + q, a.nvec - 1) * a.n + r0;
 #pragma unroll 2
-    for (int r = t0 + 32 * seg + lane; r < t1; r += 32 * nseg) {
+    for (int r = 32 * seg + lane; r < rows; r += 32 * nseg) {
       const double x = ws[r];
 #pragma unroll
       for (int q = 0; q < 8; ++q) s[q] = fma(__ldg(p[q] + r), x, s[q]);
@@ -330,32 +329,29 @@ struct CgsDots {
   }
 };
 
-// ws -= V h over the rows [t0, t1) of the chunk; upd: [js][a.rows] shared (js
-// > 1).  Ends with a barrier.
-__device__ void cgs_update(const CgsArgs& a, double* __restrict__ ws, double* __restrict__ upd, int64_t r0, int t0,
-                           int t1, const double* __restrict__ h) {
+// ws -= V h over the chunk; upd: [js][a.rows] shared, the sums of js column
+// parts.  Ends with a barrier.
+__device__ void cgs_update(const CgsArgs& a, double* __restrict__ ws, double* __restrict__ upd, int64_t r0, int rows,
+                           const double* __restrict__ h) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rb = (t1 - t0 + 31) / 32;
+  const int rb = (rows + 31) / 32;
   for (int it = warp; it < rb * a.js; it += CGS_WARPS) {
-    const int r = t0 + 32 * (it % rb) + lane, part = it / rb;
-    if (r < t1) {
+    const int r = 32 * (it % rb) + lane, part = it / rb;
+    if (r < rows) {
       const double* p = a.V + r0 + r;
       double s = 0.0;
 #pragma unroll 8
       for (int c = part; c < a.nvec; c += a.js) s = fma(__ldg(p + (int64_t)c * a.n), h[c], s);
-      if (a.js == 1) ws[r] -= s;
-      else upd[part * a.rows + r] = s;
+      upd[part * a.rows + r] = s;
     }
   }
   __syncthreads();
-  if (a.js > 1) {
-    for (int r = t0 + threadIdx.x; r < t1; r += CGS_THREADS) {
-      double t = upd[r];
-      for (int q = 1; q < a.js; ++q) t += upd[q * a.rows + r];
-      ws[r] -= t;
-    }
-    __syncthreads();
+  for (int r = threadIdx.x; r < rows; r += CGS_THREADS) {
+    double t = upd[r];
+    for (int q = 1; q < a.js; ++q) t += upd[q * a.rows + r];
+    ws[r] -= t;
   }
+  __syncthreads();
 }
 
 // sums of every CTA's partials into out[0:nout] (shared memory): every warp
@@ -389,7 +385,7 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
   __shared__ double psum[CGS_WARPS * MAXV];
   __shared__ double h1[MAXV], h2[MAXV], wn2s[1];
   double* ws = cgs_smem;               // [a.rows]
-  double* upd = cgs_smem + a.rows;     // [js][a.rows] if js > 1
+  double* upd = cgs_smem + a.rows;     // [js][a.rows]
   const int64_t r0 = (int64_t)blockIdx.x * a.rows;
   const int rows = (int)max((int64_t)0, min((int64_t)a.rows, a.n - r0));
   const int64_t stride = (int64_t)gridDim.x * MAXV;
@@ -398,24 +394,20 @@ __global__ void __launch_bounds__(CGS_THREADS, 2) cgs2_coop_kernel(CgsArgs a) {
   __syncthreads();
   {
     CgsDots d(a.nvec);
-    d.add(a, ws, r0, 0, rows);
+    d.add(a, ws, r0, rows);
     d.finish(a, psum, part);
   }
   grid.sync();
   cgs_reduce<CGS_WARPS, MAXV>(a.part, a.nvec, psum, h1);
+  cgs_update(a, ws, upd, r0, rows, h1);
   {
     CgsDots d(a.nvec);
-    const int tile = a.js > 1 ? rows : CGS_TILE;
-    for (int t0 = 0; t0 < rows; t0 += tile) {
-      const int t1 = min(rows, t0 + tile);
-      cgs_update(a, ws, upd, r0, t0, t1, h1);
-      d.add(a, ws, r0, t0, t1);
-    }
+    d.add(a, ws, r0, rows);
     d.finish(a, psum, part + stride);
   }
   grid.sync();
   cgs_reduce<CGS_WARPS, MAXV>(a.part + stride, a.nvec, psum, h2);
-  cgs_update(a, ws, upd, r0, 0, rows, h2);
+  cgs_update(a, ws, upd, r0, rows, h2);
   {
     double s = 0.0;
     for (int r = threadIdx.x; r < rows; r += CGS_THREADS) s = fma(ws[r], ws[r], s);
@@ -736,8 +728,8 @@ void Gmres::ensure(int64_t n_, int m_) {
       coop_grid = (int)std::min<int64_t>((n_ >= 1024 * (int64_t)sms ? 2 : 1) * sms, g);
       cgs_rows = (int)round_up(cdiv(n_, coop_grid), 32);
       coop_grid = (int)cdiv(n_, cgs_rows);
-      cgs_js = (int)std::min<int64_t>(CGS_JS, std::max<int64_t>(1, 4 * CGS_WARPS / (cgs_rows / 32)));
-      cgs_smem = (size_t)cgs_rows * (cgs_js > 1 ? 1 + cgs_js : 1) * sizeof(double);
+      cgs_js = (int)std::min<int64_t>(CGS_JS, std::max<int64_t>(2, 4 * CGS_WARPS / (cgs_rows / 32)));
+      cgs_smem = (size_t)cgs_rows * (1 + cgs_js) * sizeof(double);
       CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs2_coop_kernel, CGS_THREADS, cgs_smem));
       if (coop_grid > per_sm * sms) coop_grid = 0;
     }
