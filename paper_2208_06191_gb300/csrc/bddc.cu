@@ -1685,13 +1685,14 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
   C->local_bytes = lb;
   C->apply_flops = (double)lb / (double)C->esize * 2.0;
   // FP64 lists (local operators of FP64 contexts, the coarse inverse): one
-  // scratch buffer for the digits, shared by every list.  The coarsest
-  // inverse under FP32 level-2 operators keeps the FMA kernel: the hardest
-  // Newton states of the 3M-DoF P2 ventricle converge or stagnate with the
-  // last bits of the preconditioner (519 iterations, or more than 1000 in two
-  // of seven runs from states moved by 1e-13, with either kernel), the FMA
-  // kernel's bits are the ones those solves are validated with, and the
-  // inverse is small (867 unknowns: 1.9 ms of a 290 ms setup).
+  // scratch buffer for the digits, shared by every list.  The coarsest inverse
+  // under FP32 level-2 operators keeps the FMA kernel.  That is a choice about
+  // reproducibility, not about accuracy: the hardest Newton states of the 3M-DoF P2
+  // ventricle converge or stagnate with the last bits of the preconditioner
+  // (519 iterations, or more than 1000 in two of seven runs from states moved by
+  // 1e-13, with either kernel), the recorded solves of those states used the FMA
+  // kernel's bits, and the inverse is small (867 unknowns: 1.9 ms of a 290 ms
+  // setup).
   {
     std::vector<GemmList*> lists;
     if (C->esize == 8 || P->nnzb > 0)

@@ -38,10 +38,11 @@ struct GemmProb {
 };
 
 // FP32 setup GEMMs run on the tensor cores (tcgen05, split TF32) unless
-// this is cleared (cbddc_set_tensor_cores); the FP64 path always uses the
-// SIMT kernels.  tc_parts(sweep) is the number of TF32 parts per operand
-// (2 or 3) for sweep updates and for the other products, read when a
-// context is created.
+// this is cleared (cbddc_set_tensor_cores).  FP64 lists run there as integer
+// slices whatever it says (oz_gemm.cuh), but for the coarsest inverse under FP32
+// level-2 operators, which has no digit scratch and uses the CUDA cores.
+// tc_parts(sweep) is the number of TF32 parts per operand (2 or 3) for sweep
+// updates and for the other products, read when a context is created.
 bool tensor_cores_enabled();
 bool tensor_cores_for(bool sweep);  // per kind of list (sweep updates / other products)
 bool tc_sweep_ks1();                 // sweep updates accumulate one K-step per TMEM slice
