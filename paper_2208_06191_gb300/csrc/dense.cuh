@@ -399,9 +399,9 @@ struct GemmList {
       // rows as fit beside all columns, or half of the cap each
       const int64_t fit = cap / ((int64_t)oz::S * Kp * 2 + 8);
       int bm = q.M, bn = q.N;
-      if ((int64_t)q.M + q.N > fit) {
+      if (q.M + round_up(q.N, 16) > fit) {
         if (q.N > fit / 2) bn = (int)std::min<int64_t>(q.N, std::max<int64_t>(oz::BN, fit / 2 / oz::BN * oz::BN));
-        bm = (int)std::min<int64_t>(q.M, std::max<int64_t>(oz::BM, (fit - bn) / oz::BM * oz::BM));
+        bm = (int)std::min<int64_t>(q.M, std::max<int64_t>(oz::BM, (fit - round_up(bn, 16)) / oz::BM * oz::BM));
       }
       for (int m0 = 0; m0 < q.M; m0 += bm)
         for (int n0 = 0; n0 < q.N; n0 += bn) {
@@ -411,7 +411,7 @@ struct GemmList {
             oz::Batch b = oz_batches.back();
             b.Kp = std::max(b.Kp, Kp);
             b.rowsA += M;
-            b.rowsB += N;
+            b.rowsB += round_up(N, 16);
             fresh = b.bytes() > cap || b.rowsA >= INT32_MAX || b.rowsB >= INT32_MAX;
           }
           if (fresh) {
@@ -425,12 +425,12 @@ struct GemmList {
           oz::Batch& b = oz_batches.back();
           b.Kp = std::max(b.Kp, Kp);
           pr.push_back(oz::Prob{M, N, q.K, q.ldc, q.c + (int64_t)m0 * q.ldc + n0, (int)b.rowsA, (int)b.rowsB});
-          sa.push_back(oz::SplitProb{M, q.K, q.lda, (int)b.rowsA, q.ks, q.a + (int64_t)m0 * (trans_a ? 1 : q.lda),
+          sa.push_back(oz::SplitProb{M, M, q.K, q.lda, (int)b.rowsA, q.ks, q.a + (int64_t)m0 * (trans_a ? 1 : q.lda),
                                      q.ke});
-          sb.push_back(oz::SplitProb{N, q.K, q.ldb, (int)b.rowsB, -q.ks, q.b + (int64_t)n0 * (trans_b ? q.ldb : 1),
-                                     q.ke});
+          sb.push_back(oz::SplitProb{N, (int)round_up(N, 16), q.K, q.ldb, (int)b.rowsB, -q.ks,
+                                     q.b + (int64_t)n0 * (trans_b ? q.ldb : 1), q.ke});
           b.rowsA += M;
-          b.rowsB += N;
+          b.rowsB += round_up(N, 16);
           for (int k = 0; k < (int)cdiv(M, 32); ++k) ia.push_back(make_int2(i, k));
           for (int k = 0; k < (int)cdiv(N, 32); ++k) ib.push_back(make_int2(i, k));
           for (int tm = 0; tm < (int)cdiv(M, oz::BM); ++tm)

@@ -100,9 +100,12 @@ __device__ __forceinline__ void tmem_ld16i(uint32_t taddr, int* v) {
 }
 
 // ------------------------------------------------------------------- split
-// One operand of a problem: output row r (< rows) holds op(X)(r, 0:K).
+// One operand of a problem: output row r (< rows) holds op(X)(r, 0:K), and rows
+// up to out_rows hold zeros.  (op(B) is padded to the epilogue's groups of 16
+// columns, which are shifted together: with the next problem's rows there, the
+// last bits of a product would depend on it.)
 struct SplitProb {
-  int rows, K, ld;
+  int rows, out_rows, K, ld;
   int r0;       // first output row
   int ks;       // op(X)(:, k) is scaled by 2^(ks kexp[ke + k]); 0: not scaled
   int64_t off, ke;
@@ -223,7 +226,7 @@ split_kernel(const int2* __restrict__ items, const SplitProb* __restrict__ probs
     for (int w = 0; w < 8; ++w) key = max(key, keys[w][row]);
   }
   const int rw = it.y * 32 + row;  // row written
-  const bool out_in = rw < q.rows;
+  const bool out_in = rw < q.out_rows;
   // (a row of zeros takes any exponent)
   if (out_in && grp == 0) exps[q.r0 + rw] = key == KEY_NAN ? EXP_NAN : key == KEY_NONE ? 0 : key - 1022;
   __half* dst = out + (int64_t)(q.r0 + rw) * Kp + 8 * grp;
@@ -283,8 +286,10 @@ struct Maps {
 // Cost of a tile of a rank-64 update: 112 MMAs of about 70 clocks (4.1 us),
 // and beside them in the epilogue 7 float to integer conversions (16 per
 // clock) and two FP64 instructions per entry (2 per clock).  Measured: 6.3 us
-// per tile on 8192^2 x 64 (345 us, 25 TFLOP/s, 3.1 TB/s of C; the FP64 FMA
-// kernel ran at 1.1 TFLOP/s), 4.4 us per K block on 2048^2 x 768 (30 TFLOP/s).  Eight
+// per tile on 8192^2 x 64 (338 us, 25 TFLOP/s, 3.2 TB/s of C; the FP64 FMA
+// kernel ran at 1.1 TFLOP/s), 4.3 us per K block on 2048^2 x 768 (31 TFLOP/s).
+// A C whose leading dimension is no multiple of four goes entry by entry
+// (1390 us on 8192^2 x 64).  Eight
 // epilogue warps of 32 columns took 11 us per tile (two warps per scheduler do
 // not cover the latencies), and adding to C by bulk reductions in the L2 12 us
 // (they queue in front of the operand loads).
@@ -455,8 +460,7 @@ gemm_kernel(const int4* __restrict__ tiles, int ntiles, const Prob* __restrict__
       int top = 0;
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
-        // (columns past N hold products with another problem's digits)
-        const int h = n0 + q < p.N ? (int)(hi[q] >> 32) : 0;
+        const int h = (int)(hi[q] >> 32);
         top |= h ^ (h >> 31);
       }
       const int sh = max(0, 64 - 35 - __clz(top));
