@@ -1707,8 +1707,16 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
           if (g.panel) lists.push_back(g.panel.get());
         }
     }
-    int64_t need = 0;
-    for (int64_t cap = oz::kBatchBytes;;) {
+    // at most a sixteenth of what is free (vectors and the Krylov basis follow)
+    size_t left = 0, total = 0;
+    if (!lists.empty()) CB_CUDA(cudaMemGetInfo(&left, &total));
+    int64_t need = 0, cap = oz::kBatchBytes;
+    int64_t next_cap = std::min(cap, std::max((int64_t)(left / 16), oz::kMinBatchBytes));
+    for (;;) {
+      if (next_cap < cap)
+        for (auto* g : lists)
+          if (g->ntiles > 0) g->plan_oz(next_cap);
+      cap = next_cap;
       need = 0;
       for (auto* g : lists) need = std::max(need, g->oz_bytes());
       try {
@@ -1717,9 +1725,7 @@ void bddc_create(fem_problem* P, const bddc_options* opt, bddc_ctx* C) {
       } catch (const Error& e) {
         if (e.code != CBDDC_ENOMEM || cap <= oz::kMinBatchBytes) throw;
       }
-      cap = std::max(cap / 4, oz::kMinBatchBytes);
-      for (auto* g : lists)
-        if (g->ntiles > 0) g->plan_oz(cap);
+      next_cap = std::max(cap / 4, oz::kMinBatchBytes);
     }
     if (need > 0) {
       C->kexp.alloc((size_t)nke);

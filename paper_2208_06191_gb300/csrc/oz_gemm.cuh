@@ -27,10 +27,12 @@
 //   * the epilogue adds the order sums of every K block in two 64-bit
 //     integers (exact) and rounds once to FP64.
 //
-// Errors against extended precision on Gauss-Jordan sweeps of elasticity
-// matrices (Q1 and Q2 slabs, P1 ventricle, 588 to 882 unknowns): 0.9, 0.6
-// and 1.1 times those of the FP64 FMA kernel.  With six slices (54 bits) they
-// were 2.1, 2.4 and 1.1 times as large, which is why there are seven.
+// Errors against extended precision of inverses by Gauss-Jordan sweeps of
+// elasticity matrices (Q1 and Q2 slabs, P1 and P2 ventricles, 210 to 369 unknowns,
+// root mean square over five states): 0.93, 0.57, 1.03 and 0.80 times those of the
+// FP64 FMA kernel (single states: 0.4 to 1.4 times).  With six slices (54 bits)
+// single states were 2.1, 2.4 and 1.1 times as far off (Q1, Q2, P1), which is why
+// there are seven.
 //
 // The powers of two along K (Jacobi scaling) keep that so for graded matrices.
 // FMAs do not see a diagonal scaling between the operands, but entries held
@@ -560,8 +562,8 @@ struct Batch {
 
 // Digits of one batch, at most: problems share a batch while they fit, and
 // a larger one is cut into blocks of whole tiles.  A context keeps one buffer of
-// this size, or less where its products need less or the memory is short (down
-// to the second figure).  Each batch costs three launches and a last wave of
+// this size, or less where its products need less or the memory is short (a
+// sixteenth of what is free, down to the second figure).  Each batch costs three launches and a last wave of
 // tiles: the FP64 Newton step of the 48x48x12 slab (60 ms), whose E and S take 2.3
 // and 2.4 GB of digits, takes 1% longer with 1 GiB than with 2 GiB, and 2% longer
 // with 512 MiB.
