@@ -275,7 +275,10 @@ typedef struct {
   int n_primal2;               /* level-2 coarse dimension (levels = 3)     */
   int precision;
   int64_t local_bytes;         /* bytes of local operators read per apply   */
-  int64_t device_bytes;        /* device memory held by the context         */
+  int64_t device_bytes;        /* device memory held by the context: local
+                                  operators, vectors, index arrays, plans,
+                                  setup scratch, and (after its first solve)
+                                  the GMRES workspace                       */
   double setup_flops;          /* algorithmic flops of the last setup       */
   int sweep_block;             /* pivot block width of the local sweeps     */
   int tile_order;              /* tile order of the setup GEMMs             */
